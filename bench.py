@@ -51,7 +51,6 @@ UNIT = "projections/s"
 # (workload, kernel); an entry is removed whenever its kernel changes.
 MEASURED_TRAFFIC = {
     ("arm7_axis_65536", "k_project_f32+check"): 2003456,                  # read 2.00 MB, write 0
-    ("humanoid36_1048576", "k_project_group"): 238427136 + 132679936,     # read 238.4 MB, write 132.7 MB
 }
 L2_FLUSH_BYTES = 512 << 20   # > 129 MB L2
 
@@ -831,13 +830,13 @@ def measure_batch(args, name, env, sub=False):
             ach64 = fp64f / (mp * 1e-3) / 1e12
             # both pipes: the time the FP32 and FP64 work need at their peaks bounds the kernel
             t_min = max(fp32 / (peak32 * 1e12), fp64f / (peak64 * 1e12))
-            kshort = ("k_project_group" if name.startswith("humanoid") and not wl.params.cyclic else
+            kshort = ("k_project_tree" if name.startswith("humanoid") and not wl.params.cyclic else
                       "k_project_warp" if name.startswith("humanoid") else
                       "k_project_pair" if tuning and tuning.get("threads_per_config") == 2 else "k_project_f32")
             roof = {"bound": "alu", "achieved": ach32, "peak": peak32, "unit": "TFLOP/s", "frac": ach32 / peak32,
                     "traffic": MEASURED_TRAFFIC.get((wname, kshort)),
                     "kernel": kshort + {
-                        "k_project_group": " (four lanes per configuration: FP32 steps, FP64 acceptance)",
+                        "k_project_tree": " (one lane per configuration: FP32 steps, FP64 acceptance)",
                         "k_project_warp": " (warp per configuration, cyclic sweeps)",
                         "k_project_pair": " (persistent, one lane per arm: FP32 steps + FP64 acceptance)",
                         "k_project_f32": " (persistent, FP32 steps + FP64 acceptance)"}[kshort],

@@ -1,8 +1,8 @@
 // Kernel instantiations for the ProbHumanoid36Hull problem class (CoM on the
 // support polygon): the FP32 path
-// runs the group-cooperative kernel (the cyclic form: the warp kernel), the plain FP64 path and the collision
+// runs the one-lane-per-configuration tree kernel (the cyclic form: the warp kernel), the plain FP64 path and the collision
 // check the thread-per-configuration kernels.
-#include "mcp_group.cuh"
+#include "mcp_tree.cuh"
 
 namespace mcp {
 
@@ -17,10 +17,10 @@ cudaError_t launch_project<ProbHumanoid36Hull>(const HostModel &hm, const ProjCa
     if (e == cudaSuccess && c.fused_check) e = check_outputs<ProbHumanoid36Hull>(hm, c, launches);
     return e;
   }
-  // stacked form: four lanes per configuration; the cyclic form's masked
+  // stacked form: one lane per configuration; the cyclic form's masked
   // sub-steps run on the warp-per-configuration kernel
   cudaError_t e = c.cyclic ? launch_project_warp<ProbHumanoid36Hull>(hm, c, launches)
-                           : launch_project_group<ProbHumanoid36Hull>(hm, c, launches);
+                           : launch_project_tree<ProbHumanoid36Hull>(hm, c, launches);
   if (e == cudaSuccess && c.fused_check) e = check_outputs<ProbHumanoid36Hull>(hm, c, launches);
   return e;
 }

@@ -1,38 +1,15 @@
-// Group-cooperative projection for large tree problems (the 36-DoF humanoid
-// with 20 stacked equations): four lanes share one configuration, so a warp
-// advances eight configurations at once.  One warp per configuration (the
-// warp kernel) leaves most lanes idle in every sequential stage (a 20-step
-// Cholesky, the substitutions, rows 20..31 of the Gram build); four lanes
-// keep the per-configuration work almost as dense as one thread would, while
-// the configuration's Jacobian, Gram matrix and factor live in shared memory
-// instead of one thread's registers.
+// Work plan of the humanoid's Newton step on four lanes, and the layout of one
+// configuration's state under it.
 //
-// Per FP32 iteration of Alg. 2 (stacked F, inner LM form), for each group of
-// four lanes and its configuration:
-//   1. FK along the kinematic tree: every lane walks the joints of the chains
-//      it owns (limbs, assigned by longest-first scheduling) and the shared
-//      trunk (computed by every lane), storing the joint axes and origins and
-//      the mass moments m_j c_j; a prismatic chain at the root (the floating
-//      base's translations) is placed in closed form, its rotations being
-//      constant;
-//   2. subtree mass moments C_j = m_j c_j + sum over children, limbs first,
-//      then the trunk;
-//   3. residuals, constraint c on lane c mod 4 (the pose and relative-pose
-//      constraints on one code path, so that their lanes run it together);
-//      ||F|| by a group reduction;
-//   4. the structural nonzeros of J, as (joint, constraint) segments spread
-//      over the lanes;
-//   5. the Gram matrix J J^T by blocks: each lane accumulates whole row-block
-//      pairs (6x6, 2x6, 2x2) over the joints both blocks share, in registers;
-//   6. Cholesky with rows i = 4m + g on lane g (registers), column k of L
-//      exchanged through shared memory (which keeps L by columns for the
-//      back substitution); blocks of L that the symbolic factorisation
-//      proves zero (feet rows against hand columns) are skipped at compile
-//      time, in the factorisation and both substitutions;
-//   7. forward / back substitution, dq = J^T y, one refinement step
-//      (r = F - J dq - lambda y), alpha, MaxDistance, q <- q - dq.
-// Finished configurations are parked and accepted in FP64 32 at a time, one
-// per lane (the thread-level acceptance of the other kernels).
+// The plan fixes an order for every sum over joints: the limbs are assigned to
+// four lanes by longest-first scheduling and the trunk joints to the lane with
+// the fewest, the 6-row Gram blocks and refinement residuals run over the
+// joints in ascending order, and the CoM sums in one partial per lane (the
+// lane's limb joints, then its trunk joints) added pairwise.  The projection
+// kernel (one lane per configuration, mcp_tree.cuh) takes its sums in this
+// order; the host checks under tests/ compile the plan and compare.  Also
+// here: the compile-time zero pattern of the Cholesky factor and the constants
+// of the floating base's prismatic chain, which that kernel uses.
 #pragma once
 
 #include <algorithm>
@@ -606,977 +583,9 @@ struct GrpShared {
   GroupPlan<P> pl;
 };
 
-// Sum over the four lanes of a group.
-__device__ __forceinline__ float grp_sum(float v) {
-  v += __shfl_xor_sync(FULL, v, 1);
-  v += __shfl_xor_sync(FULL, v, 2);
-  return v;
-}
-
-__device__ __forceinline__ float2 lds2(const float *p) { return *reinterpret_cast<const float2 *>(p); }
-
-// Residual of constraint c (compile time) into S.F, with the data the
-// Jacobian needs; returns this constraint's squared norm.
-template <class P, int c>
-__device__ __forceinline__ float grp_residual(const ModelT<float> &m, GrpState<P> &S, const float (&tot)[3]) {
-  constexpr int kind = P::ckind(c);
-  constexpr int r0 = roff<P>(c);
-  auto &E = S.u.e;
-  const float(*Tf)[12] = reinterpret_cast<const float(*)[12]>(S.J);
-  if constexpr (kind == K_COM) {
-    const float f0 = fmaf(tot[0], m.inv_mass, -m.ctgt[c][0]);
-    const float f1 = fmaf(tot[1], m.inv_mass, -m.ctgt[c][1]);
-    S.F[r0] = f0;
-    S.F[r0 + 1] = f1;
-    return fmaf(f0, f0, f1 * f1);
-  } else if constexpr (kind == K_HULL) {
-    const float cx = tot[0] * m.inv_mass, cy = tot[1] * m.inv_mass;
-    float px, py, nx, ny;
-    constexpr int hs = grp_hslot<P>(c);
-    E.hmode[hs] = polygon_nearest<float>(m.cB[c], static_cast<int>(m.ctgt[c][0]), cx, cy, px, py, nx, ny);
-    E.hn[hs][0] = nx;
-    E.hn[hs][1] = ny;
-    const float f0 = cx - px, f1 = cy - py;
-    S.F[r0] = f0;
-    S.F[r0 + 1] = f1;
-    return fmaf(f0, f0, f1 * f1);
-  } else {
-    static_assert(kind == K_POSE || kind == K_REL, "pose-like constraint expected");
-    constexpr int ps = grp_pslot<P>(c);
-    float Pr[9], Rerr[9], G[9];
-    load_R(m.cPinv[c], Pr);
-    const V3<float> Pp = load_p(m.cPinv[c]);
-    V3<float> t, xpt;
-    constexpr int fa = P::cfa(c);
-    float Ra[9];
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-      for (int cc = 0; cc < 3; ++cc) Ra[r * 3 + cc] = Tf[fa][r * 4 + cc];
-    const V3<float> pa{Tf[fa][3], Tf[fa][7], Tf[fa][11]};
-    if constexpr (kind == K_POSE) {
-      float Qr[9], RaQ[9];
-      load_R(m.cQinv[c], Qr);
-      mul33(Ra, Qr, RaQ);
-      xpt = add_rot_t<7>(pa, Ra, load_p(m.cQinv[c]));
-      mul33(Pr, RaQ, Rerr);
-      const V3<float> tx = mulv(Pr, xpt);
-      t = {tx.x + Pp.x, tx.y + Pp.y, tx.z + Pp.z};
-#pragma unroll
-      for (int i = 0; i < 9; ++i) G[i] = Pr[i];
-    } else {
-      constexpr int fb = P::cfb(c);
-      float Rb[9];
-#pragma unroll
-      for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int cc = 0; cc < 3; ++cc) Rb[r * 3 + cc] = Tf[fb][r * 4 + cc];
-      const V3<float> pb{Tf[fb][3], Tf[fb][7], Tf[fb][11]};
-#pragma unroll
-      for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int cc = 0; cc < 3; ++cc)
-          G[r * 3 + cc] = fmaf(Pr[r * 3], Ra[cc * 3], fmaf(Pr[r * 3 + 1], Ra[cc * 3 + 1], Pr[r * 3 + 2] * Ra[cc * 3 + 2]));
-      mul33(G, Rb, Rerr);
-      const V3<float> tx = mulv(G, sub(pb, pa));
-      t = {tx.x + Pp.x, tx.y + Pp.y, tx.z + Pp.z};
-      xpt = pb;
-    }
-    const auto lg = so3_log<OpsF32, float>(Rerr);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) E.G[ps][i] = G[i];
-    E.x[ps][0] = xpt.x;
-    E.x[ps][1] = xpt.y;
-    E.x[ps][2] = xpt.z;
-    E.phi[ps][0] = lg.phi.x;
-    E.phi[ps][1] = lg.phi.y;
-    E.phi[ps][2] = lg.phi.z;
-    E.phi[ps][3] = jl_inv_beta<float>(lg.theta, lg.s, lg.c);
-    S.F[r0] = t.x;
-    S.F[r0 + 1] = t.y;
-    S.F[r0 + 2] = t.z;
-    S.F[r0 + 3] = lg.phi.x;
-    S.F[r0 + 4] = lg.phi.y;
-    S.F[r0 + 5] = lg.phi.z;
-    return fmaf(t.x, t.x, fmaf(t.y, t.y, fmaf(t.z, t.z, fmaf(lg.phi.x, lg.phi.x, fmaf(lg.phi.y, lg.phi.y, lg.phi.z * lg.phi.z)))));
-  }
-}
-
-// Residual of pose-like constraint c (run time: the pose and relative-pose
-// constraints of a stack run one code path, on their lanes at once) into
-// S.F, with the data the Jacobian needs; returns its squared norm.
-//   pose (Eq. 1):          G = P^-1_R,          R_err = G (R_a Q^-1_R),
-//                          x = p_a + R_a Q^-1_p, t = G x + P^-1_p;
-//   relative pose (Eq. 2): G = P^-1_R R_a^T,    R_err = G R_b,
-//                          x = p_b,             t = G (p_b - p_a) + P^-1_p.
-// Each product is formed with the operands the constraint's kind selects,
-// in the same order as for that kind alone.
-template <class P>
-__device__ __forceinline__ float grp_residual_pose(const ModelT<float> &m, GrpState<P> &S, const GroupPlan<P> &pl,
-                                                   int c) {
-  auto &E = S.u.e;
-  const float(*Tf)[12] = reinterpret_cast<const float(*)[12]>(S.J);
-  const bool rel = pl.crel[c] != 0;
-  const int r0 = pl.croff[c], ps = pl.pslot[c], fa = pl.cfa[c], fb = pl.cfb[c];
-  float Pr[9], Qr[9], Ra[9], Rb[9];
-  load_R(m.cPinv[c], Pr);
-  load_R(m.cQinv[c], Qr);
-  const V3<float> Pp = load_p(m.cPinv[c]);
-  const V3<float> Qp = load_p(m.cQinv[c]);
-#pragma unroll
-  for (int r = 0; r < 3; ++r)
-#pragma unroll
-    for (int cc = 0; cc < 3; ++cc) {
-      Ra[r * 3 + cc] = Tf[fa][r * 4 + cc];
-      Rb[r * 3 + cc] = Tf[fb][r * 4 + cc];
-    }
-  const V3<float> pa{Tf[fa][3], Tf[fa][7], Tf[fa][11]};
-  const V3<float> pb{Tf[fb][3], Tf[fb][7], Tf[fb][11]};
-  float X1[9], Y1[9], Z[9], X2[9], Y2[9], Rerr[9], G[9];
-#pragma unroll
-  for (int r = 0; r < 3; ++r)
-#pragma unroll
-    for (int cc = 0; cc < 3; ++cc) {
-      X1[r * 3 + cc] = rel ? Pr[r * 3 + cc] : Ra[r * 3 + cc];
-      Y1[r * 3 + cc] = rel ? Ra[cc * 3 + r] : Qr[r * 3 + cc];
-    }
-  mul33(X1, Y1, Z);  // pose: R_a Q^-1_R; relative pose: G
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    X2[i] = rel ? Z[i] : Pr[i];
-    Y2[i] = rel ? Rb[i] : Z[i];
-    G[i] = rel ? Z[i] : Pr[i];
-  }
-  mul33(X2, Y2, Rerr);
-  const V3<float> xq = add_rot_t<7>(pa, Ra, Qp);
-  const V3<float> xpt{rel ? pb.x : xq.x, rel ? pb.y : xq.y, rel ? pb.z : xq.z};
-  const V3<float> tx = mulv(G, rel ? sub(pb, pa) : xq);
-  const V3<float> t{tx.x + Pp.x, tx.y + Pp.y, tx.z + Pp.z};
-  const auto lg = so3_log<OpsF32, float>(Rerr);
-#pragma unroll
-  for (int i = 0; i < 9; ++i) E.G[ps][i] = G[i];
-  E.x[ps][0] = xpt.x;
-  E.x[ps][1] = xpt.y;
-  E.x[ps][2] = xpt.z;
-  E.phi[ps][0] = lg.phi.x;
-  E.phi[ps][1] = lg.phi.y;
-  E.phi[ps][2] = lg.phi.z;
-  E.phi[ps][3] = jl_inv_beta<float>(lg.theta, lg.s, lg.c);
-  S.F[r0] = t.x;
-  S.F[r0 + 1] = t.y;
-  S.F[r0 + 2] = t.z;
-  S.F[r0 + 3] = lg.phi.x;
-  S.F[r0 + 4] = lg.phi.y;
-  S.F[r0 + 5] = lg.phi.z;
-  return fmaf(t.x, t.x, fmaf(t.y, t.y, fmaf(t.z, t.z, fmaf(lg.phi.x, lg.phi.x, fmaf(lg.phi.y, lg.phi.y, lg.phi.z * lg.phi.z)))));
-}
-
-// Gram phase with row blocks of RA x RB rows: every lane runs its task slots;
-// each task accumulates sum_j seg(j, a) seg(j, b)^T over its joints in
-// registers and stores the lower-triangular part into S.u.A.
-template <int RA, int RB, class P>
-__device__ __forceinline__ void grp_gram_phase(const GroupPlan<P> &pl, int ph, int g, bool go, GrpState<P> &S) {
-#pragma unroll 1
-  for (int t = 0; t < pl.g_nt[ph]; ++t) {
-    const GrpTask tk = pl.gt[ph][g][t];
-    float acc[RA][RB];
-#pragma unroll
-    for (int i = 0; i < RA; ++i)
-#pragma unroll
-      for (int k = 0; k < RB; ++k) acc[i][k] = 0.f;
-    const int len = pl.g_len[ph][t];
-#pragma unroll 2
-    for (int s = 0; s < len; ++s) {
-      if (go && s < tk.n) {
-        const int j = pl.pool[tk.off + s];
-        const float *sa = S.J + pl.joff[tk.a][j];
-        const float *sb = S.J + pl.joff[tk.b][j];
-        float va[RA], vb[RB];
-#pragma unroll
-        for (int i = 0; i < RA; i += 2) {
-          const float2 v = lds2(sa + i);
-          va[i] = v.x;
-          va[i + 1] = v.y;
-        }
-#pragma unroll
-        for (int k = 0; k < RB; k += 2) {
-          const float2 v = lds2(sb + k);
-          vb[k] = v.x;
-          vb[k + 1] = v.y;
-        }
-#pragma unroll
-        for (int i = 0; i < RA; ++i)
-#pragma unroll
-          for (int k = 0; k < RB; ++k) acc[i][k] = fmaf(va[i], vb[k], acc[i][k]);
-      }
-    }
-    if (go && tk.n > 0) {
-      const int ra = pl.croff[tk.a], rb = pl.croff[tk.b];
-#pragma unroll
-      for (int i = 0; i < RA; ++i)
-#pragma unroll
-        for (int k = 0; k < RB; ++k) {
-          const int ii = ra + i, kk = rb + k;
-          if (ii >= kk) S.u.A[ii * (ii + 1) / 2 + kk] = acc[i][k];
-        }
-    }
-  }
-}
-
-// Refinement phase with row blocks of RA rows: r_a = F_a - sum_j seg(j, a) dq_j - lambda y_a.
-template <int RA, class P>
-__device__ __forceinline__ void grp_resid_phase(const GroupPlan<P> &pl, int ph, int g, bool go, float lambda,
-                                                GrpState<P> &S) {
-#pragma unroll 1
-  for (int t = 0; t < pl.r_nt[ph]; ++t) {
-    const GrpTask tk = pl.rt[ph][g][t];
-    float acc[RA];
-#pragma unroll
-    for (int i = 0; i < RA; ++i) acc[i] = 0.f;
-    const int len = pl.r_len[ph][t];
-#pragma unroll 2
-    for (int s = 0; s < len; ++s) {
-      if (go && s < tk.n) {
-        const int j = pl.pool[tk.off + s];
-        const float *sa = S.J + pl.joff[tk.a][j];
-        const float dj = S.u.s.dq[j];
-#pragma unroll
-        for (int i = 0; i < RA; i += 2) {
-          const float2 v = lds2(sa + i);
-          acc[i] = fmaf(v.x, dj, acc[i]);
-          acc[i + 1] = fmaf(v.y, dj, acc[i + 1]);
-        }
-      }
-    }
-    if (go && tk.n > 0) {
-      const int ra = pl.croff[tk.a];
-#pragma unroll
-      for (int i = 0; i < RA; ++i) S.F[ra + i] = fmaf(-lambda, S.u.s.y[ra + i], S.F[ra + i] - acc[i]);
-    }
-  }
-}
-
-// One FP32 iteration for the group's configuration.  All lanes of the warp
-// call it together (it holds warp-wide synchronisation); `act` says whether
-// this group has a configuration.  Returns true for a group whose
-// configuration leaves the FP32 loop (flags say why).
-template <class P, class A>
-__device__ __forceinline__ bool grp_iter(const A &a, const GrpTables<P> &tb, const GroupPlan<P> &pl,
-                                         GrpState<P> &S, bool act, int &it, uint32_t &fl) {
-  constexpr int K = kdim<P>(), NC = P::NC;
-  constexpr int MR = (K + GG - 1) / GG;  // rows per lane
-  const int lane = threadIdx.x & 31;
-  const int g = lane & (GG - 1);
-  const int base = lane & ~(GG - 1);
-  const ModelT<float> &m = a.m;
-  auto &E = S.u.e;
-
-  // 1. FK along the lane's schedule
-  {
-    float T[12], S0[12], S1[12];
-#pragma unroll
-    for (int e = 0; e < 12; ++e) T[e] = S0[e] = S1[e] = 0.f;
-    // the prismatic root chain in closed form: constant rotations, origins
-    // pre_c[i] + sum_{k <= i} q_k pre_a[k]
-    const int n_pre = pl.n_pre;
-    if (n_pre > 0 && act) {
-      float o0 = 0.f, o1 = 0.f, o2 = 0.f;
-#pragma unroll
-      for (int i = 0; i < GMAX_PRE; ++i) {
-        if (i < n_pre) {
-          const float qi = S.q[i];
-          o0 = fmaf(qi, tb.pre_a[i][0], o0);
-          o1 = fmaf(qi, tb.pre_a[i][1], o1);
-          o2 = fmaf(qi, tb.pre_a[i][2], o2);
-          const float x0 = tb.pre_c[i][0] + o0, x1 = tb.pre_c[i][1] + o1, x2 = tb.pre_c[i][2] + o2;
-          if (pl.fk_store[g][i]) {
-            E.zo[i][0] = tb.pre_a[i][0];
-            E.zo[i][1] = tb.pre_a[i][1];
-            E.zo[i][2] = tb.pre_a[i][2];
-            E.zo[i][3] = x0;
-            E.zo[i][4] = x1;
-            E.zo[i][5] = x2;
-            const float mi = tb.mass[i];
-            S.C(i)[0] = fmaf(mi, x0, tb.pre_mc[i][0]);
-            S.C(i)[1] = fmaf(mi, x1, tb.pre_mc[i][1]);
-            S.C(i)[2] = fmaf(mi, x2, tb.pre_mc[i][2]);
-          }
-          if (i == n_pre - 1) {
-#pragma unroll
-            for (int r = 0; r < 3; ++r) {
-#pragma unroll
-              for (int cc = 0; cc < 3; ++cc) T[r * 4 + cc] = tb.pre_R[i][r * 3 + cc];
-            }
-            T[3] = x0;
-            T[7] = x1;
-            T[11] = x2;
-          }
-        }
-      }
-    }
-#pragma unroll 1
-    for (int k = n_pre; k < pl.n_fk; ++k) {
-      const int j = pl.fk_j[g][k];
-      if (act && j >= 0) {
-        const int par = pl.fk_par[g][k];
-        if (par != 0) {  // a root or a branch point: the parent frame is not the last one
-#pragma unroll
-          for (int e = 0; e < 12; ++e) {
-            const float id = (e == 0 || e == 5 || e == 10) ? 1.f : 0.f;
-            T[e] = par == 1 ? S0[e] : (par == 2 ? S1[e] : id);
-          }
-        }
-        const float *X = tb.X[j];
-        float Lc[12];
-        const float qj = S.q[j];
-        if (tb.rev[j]) {
-          float sn, cs;
-          sincos_f32(qj, sn, cs);
-#pragma unroll
-          for (int r = 0; r < 3; ++r) {
-            Lc[r * 4] = fmaf(cs, X[r * 4], sn * X[r * 4 + 1]);
-            Lc[r * 4 + 1] = fmaf(cs, X[r * 4 + 1], -(sn * X[r * 4]));
-            Lc[r * 4 + 2] = X[r * 4 + 2];
-            Lc[r * 4 + 3] = X[r * 4 + 3];
-          }
-        } else {
-#pragma unroll
-          for (int r = 0; r < 3; ++r) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) Lc[r * 4 + c] = X[r * 4 + c];
-            Lc[r * 4 + 3] = fmaf(qj, X[r * 4 + 2], X[r * 4 + 3]);
-          }
-        }
-        {
-          float Tn[12];
-          compose34(T, Lc, Tn);
-#pragma unroll
-          for (int e = 0; e < 12; ++e) T[e] = Tn[e];
-        }
-        const int sv = pl.fk_save[g][k];
-        if (sv >= 0) {
-#pragma unroll
-          for (int e = 0; e < 12; ++e) {
-            if (sv == 0) S0[e] = T[e];
-            else S1[e] = T[e];
-          }
-        }
-        if (pl.fk_store[g][k]) {
-          E.zo[j][0] = T[2];
-          E.zo[j][1] = T[6];
-          E.zo[j][2] = T[10];
-          E.zo[j][3] = T[3];
-          E.zo[j][4] = T[7];
-          E.zo[j][5] = T[11];
-          const float *cm = tb.com[j];  // local link CoM
-          const float mj = tb.mass[j];
-#pragma unroll
-          for (int r = 0; r < 3; ++r)
-            S.C(j)[r] = mj * fmaf(T[r * 4], cm[0], fmaf(T[r * 4 + 1], cm[1], fmaf(T[r * 4 + 2], cm[2], T[r * 4 + 3])));
-          int f = -1;  // the task frame on this link, if any (one copy of the composition)
-          static_for<P::NF>([&](auto FF) {
-            if (j == P::frame_link(decltype(FF)::value)) f = decltype(FF)::value;
-          });
-          if (f >= 0) {
-            float Fx[12], To[12];
-#pragma unroll
-            for (int e = 0; e < 12; ++e) Fx[e] = tb.fX[f][e];
-            compose34(T, Fx, To);
-#pragma unroll
-            for (int e = 0; e < 12; ++e) S.J[f * 12 + e] = To[e];
-          }
-        }
-      }
-    }
-  }
-  __syncwarp();
-  // 2. subtree moments: limbs on their lanes, then the trunk on lane 0
-  float tot[3] = {0.f, 0.f, 0.f};
-  if constexpr (needs_com<P>()) {
-#pragma unroll 1
-    for (int k = 0; k < pl.n_cb; ++k) {
-      const int j = pl.cb_j[g][k];
-      if (act && j >= 0) {
-        float c0 = S.C(j)[0], c1 = S.C(j)[1], c2 = S.C(j)[2];
-#pragma unroll
-        for (int h = 0; h < GMAX_CH; ++h) {
-          const int cj = pl.child[j][h];
-          if (cj >= 0) {
-            c0 += S.C(cj)[0];
-            c1 += S.C(cj)[1];
-            c2 += S.C(cj)[2];
-          }
-        }
-        S.C(j)[0] = c0;
-        S.C(j)[1] = c1;
-        S.C(j)[2] = c2;
-      }
-    }
-    __syncwarp();
-    if (act && g == 0) {
-#pragma unroll 1
-      for (int k = 0; k < pl.n_cr; ++k) {
-        const int j = pl.cr_j[k];
-        float c0 = S.C(j)[0], c1 = S.C(j)[1], c2 = S.C(j)[2];
-#pragma unroll
-        for (int h = 0; h < GMAX_CH; ++h) {
-          const int cj = pl.child[j][h];
-          if (cj >= 0) {
-            c0 += S.C(cj)[0];
-            c1 += S.C(cj)[1];
-            c2 += S.C(cj)[2];
-          }
-        }
-        S.C(j)[0] = c0;
-        S.C(j)[1] = c1;
-        S.C(j)[2] = c2;
-      }
-    }
-    __syncwarp();
-#pragma unroll 1
-    for (int k = 0; k < pl.n_roots; ++k) {
-      const int rj = pl.roots[k];
-      tot[0] += S.C(rj)[0];
-      tot[1] += S.C(rj)[1];
-      tot[2] += S.C(rj)[2];
-    }
-  }
-  // 3. residuals: constraint c on lane c mod 4; the pose-like ones share one
-  // code path (run time), the others have their own (compile time)
-  float r2p = 0.f;
-  if constexpr (grp_npose<P>() > 0) {
-#pragma unroll 1
-    for (int c = g; c < NC; c += GG)
-      if (act && pl.pslot[c] >= 0) r2p += grp_residual_pose<P>(m, S, pl, c);
-  }
-  static_for<NC>([&](auto CC) {
-    constexpr int c = decltype(CC)::value;
-    if constexpr (!grp_pose_like<P>(c)) {
-      if (act && g == (c % GG)) r2p += grp_residual<P, c>(m, S, tot);
-    }
-  });
-  const float r2 = grp_sum(r2p);
-  bool done = false;
-  if (act) {
-    if (!(r2 <= FLT_MAX)) {
-      fl |= FL_NONFINITE;
-      done = true;
-    } else if (r2 < a.tol2 && !(fl & FL_INT_FORCE)) {
-      fl |= FL_INT_FP32CONV;
-      done = true;
-    } else if (it >= a.cap) {
-      fl |= FL_CAP;
-      done = true;
-    }
-  }
-  const bool go = act && !done;
-  __syncwarp();
-  // 4. Jacobian segments: the 2-row ones first (they read the subtree
-  // moments, which the 6-row segments overwrite)
-#pragma unroll 1
-  for (int k = 0; k < pl.n_j2; ++k) {
-    const int j = pl.j2_j[g][k];
-    if (go && j >= 0) {
-      const int c = pl.j2_c[g][k];
-      const float sg = static_cast<float>(tb.sgn[c][j]);
-      const V3<float> z{E.zo[j][0], E.zo[j][1], E.zo[j][2]};
-      const V3<float> o{E.zo[j][3], E.zo[j][4], E.zo[j][5]};
-      const bool rev = tb.rev[j] != 0;
-      const float Mj = tb.msub[j];
-      const float *Cj = S.C(j);
-      const V3<float> rr{fmaf(-Mj, o.x, Cj[0]), fmaf(-Mj, o.y, Cj[1]), fmaf(-Mj, o.z, Cj[2])};
-      const V3<float> d = cross(z, rr);
-      const float fpr = Mj * m.inv_mass;
-      float g0 = sg * (rev ? d.x * m.inv_mass : fpr * z.x);
-      float g1 = sg * (rev ? d.y * m.inv_mass : fpr * z.y);
-      if (pl.chull[c]) {  // inside: 0; on an edge: n n^T g; at a vertex: g
-        const int hs = pl.hslot[c];
-        const int hm = E.hmode[hs];
-        if (hm == 0) {
-          g0 = g1 = 0.f;
-        } else if (hm == 1) {
-          const float sd = fmaf(E.hn[hs][0], g0, E.hn[hs][1] * g1);
-          g0 = E.hn[hs][0] * sd;
-          g1 = E.hn[hs][1] * sd;
-        }
-      }
-      float *dst = S.J + pl.joff[c][j];
-      dst[0] = g0;
-      dst[1] = g1;
-    }
-  }
-  __syncwarp();
-#pragma unroll 1
-  for (int k = 0; k < pl.n_j6; ++k) {
-    const int j = pl.j6_j[g][k];
-    if (go && j >= 0) {
-      const int c = pl.j6_c[g][k];
-      const float sg = static_cast<float>(tb.sgn[c][j]);
-      const V3<float> z{E.zo[j][0], E.zo[j][1], E.zo[j][2]};
-      const V3<float> o{E.zo[j][3], E.zo[j][4], E.zo[j][5]};
-      float G[9];
-      const int ps = pl.pslot[c];
-#pragma unroll
-      for (int i = 0; i < 9; ++i) G[i] = E.G[ps][i];
-      const bool rev = tb.rev[j] != 0;
-      const V3<float> xp{E.x[ps][0], E.x[ps][1], E.x[ps][2]};
-      const V3<float> v = rev ? cross(z, sub(xp, o)) : z;
-      const V3<float> vt = mulv(G, v);
-      const V3<float> w = jl_inv_apply(V3<float>{E.phi[ps][0], E.phi[ps][1], E.phi[ps][2]}, E.phi[ps][3], mulv(G, z));
-      float *dst = S.J + pl.joff[c][j];
-      dst[0] = sg * vt.x;
-      dst[1] = sg * vt.y;
-      dst[2] = sg * vt.z;
-      dst[3] = rev ? sg * w.x : 0.f;
-      dst[4] = rev ? sg * w.y : 0.f;
-      dst[5] = rev ? sg * w.z : 0.f;
-    }
-  }
-  __syncwarp();
-  // 5. Gram blocks (overwrites the FK / residual data)
-  grp_gram_phase<6, 6>(pl, 0, g, go, S);
-  grp_gram_phase<6, 2>(pl, 1, g, go, S);
-  grp_gram_phase<2, 6>(pl, 2, g, go, S);
-  grp_gram_phase<2, 2>(pl, 3, g, go, S);
-  // diagonal blocks of 2-row constraints: every joint, over the dq partition
-  static_for<NC>([&](auto CC) {
-    constexpr int c = decltype(CC)::value;
-    if constexpr (grp_com_like<P>(c)) {
-      constexpr int r0 = roff<P>(c);
-      float s00 = 0.f, s10 = 0.f, s11 = 0.f;
-#pragma unroll 1
-      for (int k = 0; k < pl.n_dq; ++k) {
-        const int j = pl.dq_j[g][k];
-        const int o = j >= 0 ? pl.joff[c][j] : -1;
-        if (go && o >= 0) {
-          const float2 v = lds2(S.J + o);
-          s00 = fmaf(v.x, v.x, s00);
-          s10 = fmaf(v.y, v.x, s10);
-          s11 = fmaf(v.y, v.y, s11);
-        }
-      }
-      s00 = grp_sum(s00);
-      s10 = grp_sum(s10);
-      s11 = grp_sum(s11);
-      if (go && g == 0) {
-        S.u.A[r0 * (r0 + 1) / 2 + r0] = s00;
-        S.u.A[(r0 + 1) * (r0 + 2) / 2 + r0] = s10;
-        S.u.A[(r0 + 1) * (r0 + 2) / 2 + r0 + 1] = s11;
-      }
-    }
-  });
-  __syncwarp();
-  // 6. Cholesky: rows i = 4 mm + g in registers (row i has entries 0..i)
-  float L[MR][GG * MR];
-  float invd[MR];
-#pragma unroll
-  for (int mm = 0; mm < MR; ++mm) {
-    const int i = GG * mm + g;
-    const uint32_t am = pl.amask[i < K ? i : 0];
-    invd[mm] = 0.f;
-#pragma unroll
-    for (int b = 0; b < GG * (mm + 1); ++b) {
-      float v = 0.f;
-      if (go && i < K && b <= i && ((am >> b) & 1u)) v = S.u.A[i * (i + 1) / 2 + b];
-      if (b == i) v += a.lambda;
-      L[mm][b] = v;
-    }
-  }
-  __syncwarp();
-  float minpiv = FLT_MAX;
-  static_for<K>([&](auto KK) {
-    constexpr int k = decltype(KK)::value;
-    const int ow = k % GG, mk = k / GG;
-    const float piv = __shfl_sync(FULL, L[mk][k], base + ow);
-    minpiv = fminf(minpiv, piv);
-    const float ik = rsqrtf(piv);
-    float *col = S.u.s.Lc + lcol_base<K>(k);
-#pragma unroll
-    for (int mm = mk; mm < MR; ++mm) {
-      const int i = GG * mm + g;
-      if (i == k) {
-        invd[mm] = ik;
-        L[mm][k] = piv * ik;
-      } else if (i > k && i < K) {
-        L[mm][k] *= ik;
-      }
-      if (go && i >= k && i < K) col[i - k] = L[mm][k];
-    }
-    __syncwarp();
-    if (k + 1 < K) {
-      // column k below the diagonal, rows k+1 .. K-1
-      float cv[K];
-#pragma unroll
-      for (int b = k + 1; b < K; ++b) cv[b] = go ? col[b - k] : 0.f;
-      static_for<MR>([&](auto MMc) {
-        constexpr int mm = decltype(MMc)::value;
-        if constexpr (mm >= (k + 1) / GG && !l_col_block_zero<P, mm, k>()) {
-          const int i = GG * mm + g;
-          const float lik = L[mm][k];
-#pragma unroll
-          for (int b = k + 1; b < GG * (mm + 1) && b < K; ++b)
-            if (i > k && b <= i) L[mm][b] = fmaf(-lik, cv[b], L[mm][b]);
-        }
-      });
-    }
-  });
-  if (go && !(minpiv >= a.pivot)) {  // includes NaN: this configuration continues in FP64
-    fl |= FL_INT_NEEDS_F64;
-    done = true;
-  }
-  const bool go2 = act && !done;
-  int colo[MR];  // start of column 4 mm + g of L
-#pragma unroll
-  for (int mm = 0; mm < MR; ++mm) colo[mm] = pl.lcol[(GG * mm + g) < K ? GG * mm + g : 0];
-  // (L L^T)^{-1} b for rows held by the lanes (t[mm] = b_{4 mm + g})
-  auto subst = [&](float (&t)[MR]) {
-    static_for<K>([&](auto KK) {  // forward: L y = b
-      constexpr int k = decltype(KK)::value;
-      constexpr int ow = k % GG, mk = k / GG;
-      const float yk = __shfl_sync(FULL, t[mk] * invd[mk], base + ow);
-      static_for<MR>([&](auto MMc) {
-        constexpr int mm = decltype(MMc)::value;
-        if constexpr (mm >= mk && !l_col_block_zero<P, mm, k>()) {
-          const int i = GG * mm + g;
-          if (i == k) t[mm] = yk;
-          else if (i > k) t[mm] = fmaf(-L[mm][k], yk, t[mm]);
-        }
-      });
-    });
-    static_for<K>([&](auto KB) {  // back: L^T x = y, L[k][i] from column i
-      constexpr int k = K - 1 - decltype(KB)::value;
-      constexpr int ow = k % GG, mk = k / GG;
-      const float xk = __shfl_sync(FULL, t[mk] * invd[mk], base + ow);
-      static_for<MR>([&](auto MMc) {
-        constexpr int mm = decltype(MMc)::value;
-        if constexpr (mm <= mk && !l_row_seg_zero<P, k, mm>()) {
-          const int i = GG * mm + g;
-          if (i == k) {
-            t[mm] = xk;
-          } else if (i < k) {
-            // L[k][i]: row k of column i
-            const float l = go2 ? S.u.s.Lc[colo[mm] + (k - i)] : 0.f;
-            t[mm] = fmaf(-l, xk, t[mm]);
-          }
-        }
-      });
-    });
-  };
-  // dq = J^T y for the lane's dq joints (y from shared memory)
-  auto jt_y = [&]() {
-    float yv[K];
-#pragma unroll
-    for (int i = 0; i < K; ++i) yv[i] = go2 ? S.u.s.y[i] : 0.f;
-#pragma unroll 1
-    for (int k = 0; k < pl.n_dq; ++k) {
-      const int j = pl.dq_j[g][k];
-      if (go2 && j >= 0) {
-        float acc = 0.f;
-        static_for<NC>([&](auto CC) {
-          constexpr int c = decltype(CC)::value;
-          constexpr int rc = cdim(P::ckind(c));
-          constexpr int r0 = roff<P>(c);
-          const int o = pl.joff[c][j];
-          if (o >= 0) {
-#pragma unroll
-            for (int i = 0; i < rc; i += 2) {
-              const float2 v = lds2(S.J + o + i);
-              acc = fmaf(v.x, yv[r0 + i], fmaf(v.y, yv[r0 + i + 1], acc));
-            }
-          }
-        });
-        S.u.s.dq[j] = acc;
-      }
-    }
-  };
-  // y = A^{-1} F, then one refinement step with the residual from J,
-  // r = F - J (J^T y) - lambda y: y += A^{-1} r.  Both passes run the same
-  // code (a loop, not two inlined copies).
-  float t[MR], ty[MR];
-#pragma unroll
-  for (int mm = 0; mm < MR; ++mm) {
-    const int i = GG * mm + g;
-    t[mm] = (go2 && i < K) ? S.F[i] : 0.f;
-    ty[mm] = 0.f;
-  }
-#pragma unroll 1
-  for (int pass = 0; pass < 2; ++pass) {
-    subst(t);
-#pragma unroll
-    for (int mm = 0; mm < MR; ++mm) {
-      const int i = GG * mm + g;
-      ty[mm] += t[mm];
-      if (go2 && i < K) S.u.s.y[i] = ty[mm];
-    }
-    __syncwarp();
-    jt_y();
-    __syncwarp();
-    if (pass == 1) break;
-    grp_resid_phase<6>(pl, 0, g, go2, a.lambda, S);
-    static_for<NC>([&](auto CC) {  // 2-row blocks: every joint, over the dq partition
-      constexpr int c = decltype(CC)::value;
-      if constexpr (grp_com_like<P>(c)) {
-        constexpr int r0 = roff<P>(c);
-        float s0 = 0.f, s1 = 0.f;
-#pragma unroll 1
-        for (int k = 0; k < pl.n_dq; ++k) {
-          const int j = pl.dq_j[g][k];
-          const int o = j >= 0 ? pl.joff[c][j] : -1;
-          if (go2 && o >= 0) {
-            const float2 v = lds2(S.J + o);
-            const float dj = S.u.s.dq[j];
-            s0 = fmaf(v.x, dj, s0);
-            s1 = fmaf(v.y, dj, s1);
-          }
-        }
-        s0 = grp_sum(s0);
-        s1 = grp_sum(s1);
-        if (go2 && g == 0) {
-          S.F[r0] = fmaf(-a.lambda, S.u.s.y[r0], S.F[r0] - s0);
-          S.F[r0 + 1] = fmaf(-a.lambda, S.u.s.y[r0 + 1], S.F[r0 + 1] - s1);
-        }
-      }
-    });
-    __syncwarp();
-#pragma unroll
-    for (int mm = 0; mm < MR; ++mm) {
-      const int i = GG * mm + g;
-      t[mm] = (go2 && i < K) ? S.F[i] : 0.f;
-    }
-    __syncwarp();
-  }
-  // alpha, MaxDistance, update
-  float s2p = 0.f;
-#pragma unroll 1
-  for (int k = 0; k < pl.n_dq; ++k) {
-    const int j = pl.dq_j[g][k];
-    if (go2 && j >= 0) {
-      const float d = S.u.s.dq[j] * a.alpha;
-      S.u.s.dq[j] = d;
-      s2p = fmaf(d, d, s2p);
-    }
-  }
-  const float s2 = grp_sum(s2p);
-  if (go2 && a.max_step2 > 0.f && s2 > a.max_step2) {
-    fl |= FL_DIV;
-    done = true;
-  }
-  const bool go3 = act && !done;
-#pragma unroll 1
-  for (int k = 0; k < pl.n_dq; ++k) {
-    const int j = pl.dq_j[g][k];
-    if (go3 && j >= 0) S.q[j] -= S.u.s.dq[j];
-  }
-  if (go3) {
-    ++it;
-    fl &= ~FL_INT_FORCE;
-    if (!(s2 <= FLT_MAX)) {
-      fl |= FL_NONFINITE;
-      done = true;
-    }
-  }
-  __syncwarp();
-  return act && done;
-}
-
-template <class P, int W>
-__global__ void __launch_bounds__(W * 32, 1) k_project_group(const __grid_constant__ GroupArgs<P> a) {
-  constexpr int D = P::D;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  GrpShared<P> &sh = *reinterpret_cast<GrpShared<P> *>(smem_raw);
-  unsigned char *ws = smem_raw + ((sizeof(GrpShared<P>) + 15) & ~size_t(15));
-  __shared__ int s_item[W][40];  // parked configurations: < 32 + 8 (the launcher keeps totals below 2^31)
-  __shared__ uint32_t s_meta[W][40];
-  __shared__ int s_ritem[W][RETRY_CAP];  // sent back to the FP32 loop by the acceptance
-  __shared__ uint32_t s_rmeta[W][RETRY_CAP];
-  {
-    static_assert(sizeof(GrpTables<P>) % 4 == 0 && sizeof(GroupPlan<P>) % 4 == 0, "word copies");
-    const int *src = reinterpret_cast<const int *>(&a.t);
-    int *dst = reinterpret_cast<int *>(&sh.tb);
-    for (int i = threadIdx.x; i < static_cast<int>(sizeof(GrpTables<P>) / 4); i += blockDim.x) dst[i] = src[i];
-    const int *src2 = reinterpret_cast<const int *>(&a.pl);
-    int *dst2 = reinterpret_cast<int *>(&sh.pl);
-    for (int i = threadIdx.x; i < static_cast<int>(sizeof(GroupPlan<P>) / 4); i += blockDim.x) dst2[i] = src2[i];
-  }
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int wib = threadIdx.x >> 5;
-  const int g = lane & (GG - 1);
-  const int grp = lane >> 2;
-  GrpState<P> &S = *reinterpret_cast<GrpState<P> *>(ws + (wib * GCPW + grp) * grp_state_stride<P>());
-  long long qn = 0, qe = 0;  // warp-local queue [qn, qe)
-  bool more = true;
-  bool act = false;
-  long long item = 0;
-  int it = 0;
-  uint32_t fl = 0;
-  int pend = 0;
-  int nret = 0;  // warp-uniform count of configurations to retry in FP32
-  const unsigned lead = 0x11111111u;  // lane 0 of every group
-  while (true) {
-    // refill idle groups (decided by each group's lane 0, shared by the
-    // group): retries first, then new work
-    const unsigned idle = __ballot_sync(FULL, !act) & lead;
-    if (idle != 0u && (nret > 0 || qn < qe || more)) {
-      const int n_idle = __popc(idle);
-      const int from_r = n_idle < nret ? n_idle : nret;
-      const int need = n_idle - from_r;
-      const long long avail = qe - qn;
-      long long b0 = 0, b1 = 0;
-      if (need > 0 && avail < need && more) {
-        unsigned long long b = 0;
-        if (lane == 0) b = atomicAdd(a.counter, static_cast<unsigned long long>(a.chunk));
-        b = __shfl_sync(FULL, b, 0);
-        if (static_cast<long long>(b) >= a.total) {
-          more = false;
-        } else {
-          b0 = static_cast<long long>(b);
-          b1 = b0 + a.chunk < a.total ? b0 + a.chunk : a.total;
-        }
-      }
-      const int rank_all = __popc(idle & ((1u << (grp * GG)) - 1u));
-      if (!act) {
-        if (rank_all < from_r) {  // one more FP32 step from the parked iterate
-          const int pos = nret - 1 - rank_all;
-          item = s_ritem[wib][pos];
-          const uint32_t meta = s_rmeta[wib][pos];
-          it = static_cast<int>(meta & 0xffu);
-          fl = ((meta >> 8) & ~(FL_INT_FP32CONV | FL_INT_NEEDS_F64)) | FL_INT_FORCE;
-          act = true;
-          for (int j = g; j < D; j += GG) S.q[j] = MCP_CHK(item, a.ld_out) ? a.q_out[j * a.ld_out + item] : 0.f;
-        } else {
-          const int rank = rank_all - from_r;
-          long long cand = -1;
-          if (rank < avail) cand = qn + rank;
-          else if (rank - avail < b1 - b0) cand = b0 + (rank - avail);
-          if (cand >= 0) {
-            item = cand;
-            act = true;
-            it = 0;
-            fl = 0;
-            for (int j = g; j < D; j += GG) S.q[j] = MCP_CHK(item, a.src.ld) ? a.src.q[j * a.src.ld + item] : 0.f;
-          }
-        }
-      }
-      nret -= from_r;
-      const long long used_old = need < avail ? need : avail;
-      if (b1 > b0) {
-        const long long rest = need - used_old;
-        qn = b0 + (rest < b1 - b0 ? rest : b1 - b0);
-        qe = b1;
-      } else {
-        qn += used_old;
-      }
-    }
-    __syncwarp();
-    const bool done = grp_iter<P>(a, sh.tb, sh.pl, S, act, it, fl);
-    // park finished configurations
-    const unsigned fin = __ballot_sync(FULL, done) & lead;
-    if (fin != 0u) {
-      if (done) {
-        if (MCP_CHK(item, a.ld_out))
-          for (int j = g; j < D; j += GG) a.q_out[j * a.ld_out + item] = S.q[j];
-        if (g == 0) {
-          const int pos = pend + __popc(fin & ((1u << lane) - 1u));
-          s_item[wib][pos] = static_cast<int>(item);
-          s_meta[wib][pos] = static_cast<uint32_t>(it) | (fl << 8);
-        }
-        act = false;
-      }
-      pend += __popc(fin);
-      __syncwarp();
-    }
-    const bool drained = !__any_sync(FULL, act) && qn >= qe && !more && nret == 0;
-    // FP64 acceptance, one configuration per lane, 32 at a time; a failed
-    // acceptance with steps left goes back to the FP32 loop
-    if (pend >= 32 || (drained && pend > 0)) {
-      const int take = pend < 32 ? pend : 32;
-      const bool room = nret + take <= RETRY_CAP;
-      bool retry = false;
-      long long it_item = 0;
-      uint32_t meta = 0;
-      if (lane < take) {
-        const int pos = pend - take + lane;
-        meta = s_meta[wib][pos];
-        it_item = s_item[wib][pos];
-        retry = accept_one<P, FORM_STACKED>(a, it_item, static_cast<int>(meta & 0xffu), meta >> 8, room);
-      }
-      const unsigned rm = __ballot_sync(FULL, retry);
-      __syncwarp();
-      if (retry) {
-        const int rp = nret + __popc(rm & ((1u << lane) - 1u));
-        s_ritem[wib][rp] = static_cast<int>(it_item);
-        s_rmeta[wib][rp] = meta;
-      }
-      nret += __popc(rm);
-      pend -= take;
-      __syncwarp();
-    }
-    if (drained && pend == 0 && nret == 0) break;
-  }
-}
-
 template <class P>
 size_t group_smem_bytes(int W) {
   return ((sizeof(GrpShared<P>) + 15) & ~size_t(15)) + static_cast<size_t>(W) * GCPW * grp_state_stride<P>();
-}
-
-template <class P>
-cudaError_t launch_project_group(const HostModel &hm, const ProjCall &c, int *launches) {
-  static_assert(grp_supported<P>(), "the group kernel takes trees with pose-like and CoM-like constraints");
-  if (c.total <= 0) return cudaSuccess;
-  if (c.precision == 1 || c.segments || c.outer || c.cyclic) return cudaErrorNotSupported;
-  if (c.total > 0x7fffffffLL) return cudaErrorInvalidValue;  // parked indices are 32-bit
-  constexpr int W = 11;  // one block per SM: 88 configurations, bounded by shared memory
-  struct Planned {
-    GroupPlan<P> plan;
-    bool ok;
-  };
-  static const Planned pp = [] {  // once per class (thread-safe initialisation)
-    Planned h{};
-    h.ok = make_group_plan<P>(h.plan, nullptr);
-    return h;
-  }();
-  if (!pp.ok) return cudaErrorNotSupported;
-  GroupArgs<P> a;
-  cudaError_t err = cudaMemsetAsync(c.counter, 0, sizeof(unsigned long long), c.stream);
-  if (err != cudaSuccess) return err;
-  a.m = hm.m32;
-  a.t = make_grp_tables<P>(hm.m32, hm.m64);
-  a.pl = pp.plan;
-  a.m64 = hm.d_m64;
-  a.tab = hm.d_tab;
-  a.src = BatchSrc<float>{static_cast<const float *>(c.q_in), c.ld_in};
-  a.q_out = static_cast<float *>(c.q_out);
-  a.ld_out = c.ld_out;
-  a.flags = c.flags;
-  a.iters = c.iters;
-  a.resid = c.resid;
-  a.counter = c.counter;
-  a.total = c.total;
-  a.chunk = 16;
-  a.cap = c.cap;
-  a.tol2 = static_cast<float>(c.tol * c.tol);
-  a.lambda = static_cast<float>(c.lambda);
-  a.max_step2 = c.max_step > 0 ? static_cast<float>(c.max_step * c.max_step) : 0.f;
-  a.pivot = static_cast<float>(c.pivot);
-  a.tol2_64 = c.tol * c.tol;
-  a.lambda64 = c.lambda;
-  a.alpha = static_cast<float>(c.alpha);
-  auto kern = k_project_group<P, W>;
-  const size_t smem = group_smem_bytes<P>(W);
-  err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (err != cudaSuccess) return err;
-  int per_sm = 0;
-  err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, W * 32, smem);
-  if (err != cudaSuccess) return err;
-  if (per_sm < 1) return cudaErrorNotSupported;
-  long long blocks = static_cast<long long>(hm.sm_count) * per_sm;
-  const long long need = (c.total + static_cast<long long>(GCPW) * W - 1) / (static_cast<long long>(GCPW) * W);
-  if (blocks > need) blocks = need;
-  kern<<<static_cast<unsigned>(blocks), W * 32, smem, c.stream>>>(a);
-  *launches += 1;
-  return cudaGetLastError();
 }
 
 }  // namespace mcp
