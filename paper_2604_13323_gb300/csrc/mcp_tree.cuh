@@ -10,20 +10,24 @@
 // than the instruction cache holds.  (Four lanes per configuration, with the
 // Jacobian, Gram matrix and factor in shared memory, took 16,000
 // warp-instructions per iteration for 8 configurations: 20.7 ms for 1,048,576
-// configurations, 667 us for 4,099 and 410 us for 32, against 8.5 ms, 330 us
+// configurations, 667 us for 4,099 and 410 us for 32, against 7.2 ms, 330 us
 // and 150 us here.)  Layout:
 //   * shared memory per configuration: 129 float2 (TREE_PAIRS), lane-major
 //     (pair e of lane l at [e * 32 + l]: conflict-free 64-bit accesses at
 //     immediate offsets); seven warps of 32 configurations fill an SM's 227 KB;
 //   * the two legs, and the two arms, run the same code in a loop over the
 //     side (half the instruction footprint);
-//   * the block's warps go through an iteration in step: a barrier between its
-//     phases (TREE_SYNCS of them) keeps them within the same few KB of code, so
-//     that one fetch serves all seven.  Without the barriers the warps fetch
-//     seven places at once: 13.0 ms instead of 8.5 ms for 1,048,576;
-//   * the FP64 acceptance is taken by the block's warps together, when one of
-//     them has 32 configurations waiting (those with at least TREE_ACCEPT_MIN
-//     take part), so that no barrier waits for a single warp's FP64 pass;
+//   * warps go through an iteration in step: a barrier between its phases
+//     (TREE_SYNCS of them) keeps them within the same few KB of code, so that
+//     one fetch serves several.  Without barriers the warps fetch seven places
+//     at once: 13.0 ms instead of 8.5 ms for 1,048,576;
+//   * in two teams, of the first TREE_TEAM warps and the rest (one warp of each
+//     on a scheduler): a team takes its FP64 acceptances together, when one of
+//     its warps has 32 configurations waiting (those with at least
+//     TREE_ACCEPT_MIN take part), while the other team steps on in FP32.  Up to
+//     96 configurations wait per warp, and a token lets one team at a time
+//     accept: the teams settle in opposite phases instead of sharing the FP64
+//     unit and then leaving it idle together (8.5 -> 7.2 ms for 1,048,576);
 //   * the floating base's prismatic joints have constant Jacobian columns:
 //     these, and their share of the Gram matrix, are kernel parameters.
 //
@@ -272,6 +276,21 @@ __device__ __forceinline__ void unpack6(const float2 (&v)[3], float (&f)[6]) {
   }
 }
 
+// Warps of a block that go through the iterations in step with one another.
+struct TreeTeam {
+  int id, threads;  // named barrier and the number of threads that meet at it
+  __device__ __forceinline__ void sync() const { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
+  __device__ __forceinline__ bool any(bool v) const {
+    int r;
+    asm volatile(
+        "{\n .reg .pred p, o;\n setp.ne.s32 p, %3, 0;\n bar.red.or.pred o, %1, %2, p;\n selp.s32 %0, 1, 0, o;\n}"
+        : "=r"(r)
+        : "r"(id), "r"(threads), "r"(static_cast<int>(v))
+        : "memory");
+    return r != 0;
+  }
+};
+
 // Barriers of one iteration after its stopping test (before the hands' Gram
 // block, the feet's, the Cholesky factorisation and each solve pass).
 constexpr int TREE_SYNCS = 5;
@@ -281,7 +300,7 @@ constexpr int TREE_SYNCS = 5;
 // returns true when the configuration leaves the FP32 loop (flags say why).
 // Every warp of the block calls it (it holds block-wide barriers).
 template <class P, class A>
-__device__ __forceinline__ bool tree_iter(const A &a, float2 *__restrict__ sm, float (&q)[P::D], bool act, int &it,
+__device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float2 *__restrict__ sm, float (&q)[P::D], bool act, int &it,
                                           uint32_t &fl) {
   static_assert(tree_layout_matches<P>(), "not the humanoid tree");
   constexpr int K = kdim<P>();
@@ -411,7 +430,7 @@ __device__ __forceinline__ bool tree_iter(const A &a, float2 *__restrict__ sm, f
       for (int i = 0; i < 6; ++i) F[6 + i] = f6[i];
     }
   }
-  __syncthreads();
+  team.sync();
   // arms: FK, CoM columns, axes and origins into the segments' slots
   float Ra[9], Rb[9];
   V3<float> pa, pb{0.f, 0.f, 0.f};
@@ -447,7 +466,7 @@ __device__ __forceinline__ bool tree_iter(const A &a, float2 *__restrict__ sm, f
     if (s == 0) Carm[0] = C[0];
     else Carm[1] = C[0];
   }
-  __syncthreads();
+  team.sync();
   // the hands' relative pose: G = P^-1_R R_a^T, R_err = G R_b, t = G (p_b - p_a) + P^-1_p
   float G[9];
   TreePose eh;
@@ -516,10 +535,10 @@ __device__ __forceinline__ bool tree_iter(const A &a, float2 *__restrict__ sm, f
   }
   const bool go = act && !done;
   if (!__any_sync(FULL, go)) {  // nothing to solve in this warp: only the barriers that follow
-    for (int i = 0; i < TREE_SYNCS; ++i) __syncthreads();
+    for (int i = 0; i < TREE_SYNCS; ++i) team.sync();
     return done;
   }
-  __syncthreads();
+  team.sync();
   float2 jc[3];  // CoM columns of the prismatic joints
 #pragma unroll
   for (int i = 0; i < 3; ++i) jc[i] = make_float2(a.t.jc[i][0], a.t.jc[i][1]);
@@ -579,7 +598,7 @@ __device__ __forceinline__ bool tree_iter(const A &a, float2 *__restrict__ sm, f
       L[tri(19, 12 + i)] = CH[6 + i];
     }
   }
-  __syncthreads();
+  team.sync();
   // feet: diagonal blocks, right against left, CoM rows
   {
 #pragma unroll
@@ -679,7 +698,7 @@ __device__ __forceinline__ bool tree_iter(const A &a, float2 *__restrict__ sm, f
     L[tri(19, 18)] = __fadd_rn(__fadd_rn(p[0][1], p[1][1]), __fadd_rn(p[2][1], p[3][1]));
     L[tri(19, 19)] = __fadd_rn(__fadd_rn(p[0][2], p[1][2]), __fadd_rn(p[2][2], p[3][2]));
   }
-  __syncthreads();
+  team.sync();
   // Cholesky, right-looking, on the structural nonzeros
   float invd[K];
   float minpiv = FLT_MAX;
@@ -724,7 +743,7 @@ __device__ __forceinline__ bool tree_iter(const A &a, float2 *__restrict__ sm, f
   for (int i = 0; i < 3; ++i) db[i] = 0.f;
 #pragma unroll 1
   for (int pass = 0; pass < 2; ++pass) {
-    __syncthreads();
+    team.sync();
     static_for<K>([&](auto KK) {  // forward: L y = b
       constexpr int k = decltype(KK)::value;
       t[k] = __fmul_rn(t[k], invd[k]);
@@ -912,9 +931,9 @@ __device__ __forceinline__ bool tree_iter(const A &a, float2 *__restrict__ sm, f
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) q[TR_WAIST + i] = __fadd_rn(q[TR_WAIST + i], -at(TP_UP + i).x);
-#pragma unroll 2
+#pragma unroll
     for (int l = 0; l < 2 * TR_LEG; ++l) q[TR_LEG0 + l] = __fadd_rn(q[TR_LEG0 + l], -at(TP_LIMB + 4 * l).x);
-#pragma unroll 2
+#pragma unroll
     for (int l = 0; l < 2 * TR_ARM; ++l) q[TR_ARM0 + l] = __fadd_rn(q[TR_ARM0 + l], -at(TP_ARM + 4 * l).x);
     ++it;
     fl &= ~FL_INT_FORCE;
@@ -927,12 +946,16 @@ __device__ __forceinline__ bool tree_iter(const A &a, float2 *__restrict__ sm, f
 }
 
 // Persistent projection, one configuration per lane.  Configurations that
-// left the FP32 loop wait in registers (two per lane: the pending list's
-// positions lane and lane + 32) until 32 are there for a full warp of FP64
-// acceptances; those sent back for another FP32 step wait likewise (one per
-// lane).  A 32-word scratch per warp routes them.
+// left the FP32 loop wait in registers (TREE_SLOTS per lane: the pending
+// list's positions lane, lane + 32, ...) until 32 are there for a full warp of
+// FP64 acceptances; those sent back for another FP32 step wait likewise (one
+// per lane).  A 32-word scratch per warp routes them.  An acceptance always
+// runs once a warp could not hold another iteration's 32 configurations, or
+// has nothing else to do, with or without the token.
 constexpr int TREE_WARPS = 7;
+constexpr int TREE_TEAM = 4;
 constexpr int TREE_ACCEPT_MIN = 20;
+constexpr int TREE_SLOTS = 3;
 template <class P>
 __host__ __device__ constexpr size_t tree_smem_bytes(int warps) {
   return static_cast<size_t>(warps) * 32 * (TREE_PAIRS * sizeof(float2) + sizeof(int));
@@ -945,15 +968,20 @@ __global__ void __launch_bounds__(TREE_WARPS * 32, 1) k_project_tree(const __gri
   const int wib = threadIdx.x >> 5;
   float2 *sm = reinterpret_cast<float2 *>(smem_raw) + wib * TREE_PAIRS * 32 + lane;
   int *route = reinterpret_cast<int *>(smem_raw + (blockDim.x >> 5) * TREE_PAIRS * 32 * sizeof(float2)) + wib * 32;
+  __shared__ int fp64_taken;
+  if (threadIdx.x == 0) fp64_taken = 0;
+  __syncthreads();
+  const int warps = blockDim.x >> 5, team0 = wib < TREE_TEAM ? 0 : TREE_TEAM;  // first warp of the team
+  const TreeTeam team{1 + (team0 > 0), 32 * (team0 > 0 ? warps - TREE_TEAM : min(warps, TREE_TEAM))};
   long long qn = 0, qe = 0;  // warp-local queue [qn, qe)
   bool more = true;
   bool act = false;
   int item = 0;
   int it = 0;
   uint32_t fl = 0;
-  int pend = 0, nret = 0;                    // warp-uniform
-  int p_item[2] = {0, 0}, p_meta[2] = {0, 0};  // pending positions lane, lane + 32
-  int r_item = 0, r_meta = 0;                // retry position lane
+  int pend = 0, nret = 0;                                    // warp-uniform
+  int p_item[TREE_SLOTS] = {}, p_meta[TREE_SLOTS] = {};  // pending positions lane, lane + 32, ...
+  int r_item = 0, r_meta = 0;                              // retry position lane
   float q[D];
 #pragma unroll 1
   for (int j = 0; j < D; ++j) q[j] = 0.f;
@@ -1005,7 +1033,7 @@ __global__ void __launch_bounds__(TREE_WARPS * 32, 1) k_project_tree(const __gri
         if (src) {
           act = true;
           const bool ok = MCP_CHK(item, ld);
-#pragma unroll 6
+#pragma unroll
           for (int j = 0; j < D; ++j) q[j] = ok ? src[j * ld + item] : 0.f;
         }
       }
@@ -1019,28 +1047,33 @@ __global__ void __launch_bounds__(TREE_WARPS * 32, 1) k_project_tree(const __gri
         qn += used_old;
       }
     }
-    __syncthreads();
-    const bool done = tree_iter<P>(a, sm, q, act, it, fl);
+    bool done = false;
+    if (team.any(act)) done = tree_iter<P>(a, team, sm, q, act, it, fl);
     // park finished configurations
     const unsigned fin = __ballot_sync(FULL, done);
     if (fin != 0u) {
       const int nf = __popc(fin), rank = __popc(fin & ((1u << lane) - 1u));
       if (done) {
         if (MCP_CHK(item, a.ld_out)) {
-#pragma unroll 6
+#pragma unroll
           for (int j = 0; j < D; ++j) a.q_out[j * a.ld_out + item] = q[j];
         }
         route[rank] = item;
       }
       __syncwarp();
-      const int s0 = lane - pend, s1 = lane + 32 - pend;  // ranks that land on this lane's positions
-      if (s0 >= 0 && s0 < nf) p_item[0] = route[s0];
-      if (s1 >= 0 && s1 < nf) p_item[1] = route[s1];
+#pragma unroll
+      for (int k = 0; k < TREE_SLOTS; ++k) {  // the rank that lands on this lane's position k
+        const int r = lane + 32 * k - pend;
+        if (r >= 0 && r < nf) p_item[k] = route[r];
+      }
       __syncwarp();
       if (done) route[rank] = static_cast<int>(static_cast<uint32_t>(it) | (fl << 8));
       __syncwarp();
-      if (s0 >= 0 && s0 < nf) p_meta[0] = route[s0];
-      if (s1 >= 0 && s1 < nf) p_meta[1] = route[s1];
+#pragma unroll
+      for (int k = 0; k < TREE_SLOTS; ++k) {
+        const int r = lane + 32 * k - pend;
+        if (r >= 0 && r < nf) p_meta[k] = route[r];
+      }
       __syncwarp();
       if (done) act = false;
       pend += nf;
@@ -1048,15 +1081,25 @@ __global__ void __launch_bounds__(TREE_WARPS * 32, 1) k_project_tree(const __gri
     const bool drained = !__any_sync(FULL, act) && qn >= qe && !more && nret == 0;
     // FP64 acceptance, one configuration per lane, 32 at a time; a failed
     // acceptance with steps left goes back to the FP32 loop
-    const bool accept = __syncthreads_or(pend >= 32 || (drained && pend > 0));
+    bool accept = false, token = false;
+    if (team.any(pend >= 32 || (drained && pend > 0))) {
+      if (wib == team0 && lane == 0) token = atomicCAS(&fp64_taken, 0, 1) == 0;
+      accept = team.any(token || pend > 32 * (TREE_SLOTS - 1) || drained);
+    }
     if (accept && pend > 0 && (pend >= TREE_ACCEPT_MIN || drained)) {
       const int take = pend < 32 ? pend : 32;
       const bool room = nret + take <= 32;
       const int pos = pend - take + lane;
-      const int i0 = __shfl_sync(FULL, p_item[0], pos & 31), i1 = __shfl_sync(FULL, p_item[1], pos & 31);
-      const int m0 = __shfl_sync(FULL, p_meta[0], pos & 31), m1 = __shfl_sync(FULL, p_meta[1], pos & 31);
-      const int it_item = pos < 32 ? i0 : i1;
-      const uint32_t meta = static_cast<uint32_t>(pos < 32 ? m0 : m1);
+      int it_item = 0, im = 0;
+#pragma unroll
+      for (int k = 0; k < TREE_SLOTS; ++k) {
+        const int vi = __shfl_sync(FULL, p_item[k], pos & 31), vm = __shfl_sync(FULL, p_meta[k], pos & 31);
+        if ((pos >> 5) == k) {
+          it_item = vi;
+          im = vm;
+        }
+      }
+      const uint32_t meta = static_cast<uint32_t>(im);
       bool retry = false;
       if (lane < take) retry = accept_one<P, FORM_STACKED>(a, it_item, static_cast<int>(meta & 0xffu), meta >> 8, room);
       const unsigned rmask = __ballot_sync(FULL, retry);
@@ -1074,7 +1117,9 @@ __global__ void __launch_bounds__(TREE_WARPS * 32, 1) k_project_tree(const __gri
       }
       pend -= take;
     }
-    if (__syncthreads_and(drained && pend == 0 && nret == 0)) break;
+    const bool left = team.any(!(drained && pend == 0 && nret == 0));
+    if (token) atomicExch(&fp64_taken, 0);
+    if (!left) break;
   }
 }
 
