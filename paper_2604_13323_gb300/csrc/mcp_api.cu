@@ -175,9 +175,9 @@ __global__ void k_sincos_table(double2 *tab) {
     double s, c;
     sincospi(static_cast<double>(k) / 128.0, &s, &c);
     tab[k] = make_double2(s, c);
-  } else if (k < SPLIT_TAB_OFF + 2 * SPLIT_TAB_HALF + 1) {  // (sin, cos)(m / 512), m = -2048..2048
+  } else if (k < SPLIT_TAB_OFF + 2 * SPLIT_TAB_HALF + 1) {  // (sin, cos)(m / 1024), m = -4096..4096
     double s, c;
-    sincos(static_cast<double>(k - SPLIT_TAB_OFF - SPLIT_TAB_HALF) / 512.0, &s, &c);
+    sincos(static_cast<double>(k - SPLIT_TAB_OFF - SPLIT_TAB_HALF) / static_cast<double>(SPLIT_TAB_PER_RAD), &s, &c);
     tab[k] = make_double2(s, c);
   }
 }
@@ -677,6 +677,9 @@ void fill_robot_model(const RobotHost &r, ModelT<T> &m) {
     for (int i = 0; i < 12; ++i) m.X[j][i] = static_cast<T>(r.X[12 * j + i]);
     m.mass[j] = static_cast<T>(r.mass[j]);
     for (int i = 0; i < 3; ++i) m.com[j][i] = static_cast<T>(r.com[3 * j + i]);
+    // tested so that a value that is not finite counts as nonzero
+    for (int i = 0; i < 3; ++i) m.com_nz[j] |= static_cast<uint8_t>(m.com[j][i] == T(0) ? 0 : 1 << i);
+    m.com_nz[j] |= static_cast<uint8_t>(m.mass[j] == T(0) ? 0 : 8);
     m.lower[j] = bound_up<T>(r.lower[j]);
     m.upper[j] = bound_down<T>(r.upper[j]);
   }
@@ -694,6 +697,9 @@ void fill_constraints(const ResolveOut &ro, const std::vector<ConsHost> &cons, i
       m.cB[c][i] = static_cast<T>(ro.B[c][i]);
     }
     for (int i = 0; i < 3; ++i) m.ctgt[c][i] = static_cast<T>(ro.tgt[c][i]);
+    bool id = true;
+    for (int i = 0; i < 12; ++i) id = id && ro.Qinv[c][i] == (i == 0 || i == 5 || i == 10 ? 1.0 : 0.0);
+    m.cq_id[c] = id ? 1 : 0;
   }
   for (int j = 0; j < nj; ++j) m.msub[j] = static_cast<T>(ro.msub[j]);
   m.inv_mass = static_cast<T>(ro.inv_mass);

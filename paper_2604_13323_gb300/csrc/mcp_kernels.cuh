@@ -12,6 +12,7 @@
 
 #include <math_constants.h>
 
+#include "mcp_accept.cuh"
 #include "mcp_device.cuh"
 #include "mcp_internal.h"
 #include "mcp_problems.cuh"
@@ -633,104 +634,6 @@ __device__ __forceinline__ bool cyclic_iter_f32(const A &a, float (&q)[P::D], in
 // ---------------------------------------------------------------------------
 // FP64 pieces used by the acceptance pass.
 // ---------------------------------------------------------------------------
-template <class P>
-__host__ __device__ constexpr bool axis_only() {
-  for (int c = 0; c < P::NC; ++c)
-    if (P::ckind(c) != K_AXIS) return false;
-  return true;
-}
-template <class P>
-__host__ __device__ constexpr int chain_len(int link) {
-  int n = 0;
-  for (int l = link; l >= 0; l = P::parent(l)) ++n;
-  return n;
-}
-template <class P>
-__host__ __device__ constexpr int chain_at(int link, int k) {  // k-th joint from `link` towards the root
-  int l = link;
-  for (int i = 0; i < k; ++i) l = P::parent(l);
-  return l;
-}
-// v <- R v for a fixed rotation given by its code (signed permutation: no arithmetic) or dense
-template <int CODE>
-__device__ __forceinline__ V3<double> xrot_apply(const double *X, V3<double> v) {
-  if constexpr (CODE == XR_GENERIC) {
-    return {fma(X[0], v.x, fma(X[1], v.y, X[2] * v.z)), fma(X[4], v.x, fma(X[5], v.y, X[6] * v.z)),
-            fma(X[8], v.x, fma(X[9], v.y, X[10] * v.z))};
-  } else {
-    double o[3] = {0.0, 0.0, 0.0};
-    const double in[3] = {v.x, v.y, v.z};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) o[xr_perm(CODE, k)] = xr_neg(CODE, k) ? -in[k] : in[k];
-    return {o[0], o[1], o[2]};
-  }
-}
-
-// Squared FP64 residual of axis-alignment constraints: only the frame's z axis
-// enters F, so one vector is carried from the frame to the root,
-//   z = X_0 Rz(q_0) ... X_l Rz(q_l) Xf e_z,
-// at 4 FP64 operations per revolute joint (plus its sin/cos) instead of a
-// full rotation product.  A revolute root joint whose axis is world z (X_0
-// without rotation) turns z about world z, which leaves z.x^2 + z.y^2 = |F|^2
-// unchanged: its rotation is skipped.
-template <class P>
-__host__ __device__ constexpr bool norm_invariant_root(int j) {
-  return P::parent(j) < 0 && P::jtype(j) == REV && P::xrot(j) == XR_IDENTITY;
-}
-template <class P, class Ops, typename Q>
-__device__ __forceinline__ double axis_residual2_f64(const Ops &ops, const ModelT<double> &m, const Q (&q)[P::D]) {
-  double r2 = 0.0;
-  static_for<P::NC>([&](auto CC) {
-    constexpr int c = decltype(CC)::value;
-    constexpr int f = P::cfa(c);
-    constexpr int l = P::frame_link(f);
-    V3<double> v = xrot_apply<P::frot(f)>(m.fX[f], V3<double>{0.0, 0.0, 1.0});
-    static_for<chain_len<P>(l)>([&](auto KK) {
-      constexpr int j = chain_at<P>(l, decltype(KK)::value);
-      if constexpr (norm_invariant_root<P>(j)) {
-        return;
-      } else if constexpr (P::jtype(j) == REV) {
-        double sn, cs;
-        ops.sincos(q[j], sn, cs);
-        v = {fma(cs, v.x, -(sn * v.y)), fma(sn, v.x, cs * v.y), v.z};
-      }
-      v = xrot_apply<P::xrot(j)>(m.X[j], v);
-    });
-    r2 = fma(v.x, v.x, fma(v.y, v.y, r2));
-  });
-  return r2;
-}
-
-template <class P, class Ops>
-__device__ __forceinline__ double residual2_f64(const Ops &ops, const ModelT<double> &m,
-                                                const double (&q)[P::D]) {
-  if constexpr (axis_only<P>()) return axis_residual2_f64<P>(ops, m, q);
-  constexpr int K = kdim<P>();
-  Kin<P, double> k;
-  if constexpr (needs_fk<P>()) fk<P, needs_pos<P>()>(ops, m, q, k);
-  double F[K];
-  Eval<P, double> e;
-  residual<P, Ops, double, false>(m, q, k, F, e);
-  double r2 = 0.0;
-#pragma unroll
-  for (int i = 0; i < K; ++i) r2 = fma(F[i], F[i], r2);
-  return r2;
-}
-
-// The same for an FP32 configuration (the acceptance of an FP32 iterate): the
-// axis form takes the FP32 angles straight into the split sin/cos.
-template <class P, class Ops>
-__device__ __forceinline__ double residual2_f64(const Ops &ops, const ModelT<double> &m, const float (&q)[P::D]) {
-  if constexpr (axis_only<P>()) {
-    return axis_residual2_f64<P>(ops, m, q);
-  } else {
-    double qd[P::D];
-#pragma unroll
-    for (int j = 0; j < P::D; ++j) qd[j] = static_cast<double>(q[j]);
-    return residual2_f64<P>(ops, m, qd);
-  }
-}
-
 // One LM step entirely in FP64 at q (the re-solve of a badly conditioned
 // system).  J and the factorisation live in local memory (runtime-indexed
 // loops) so that this rare path does not raise the register budget of the
