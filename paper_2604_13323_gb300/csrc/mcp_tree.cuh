@@ -5,29 +5,33 @@
 // registers, so no stage of the Newton step has idle lanes, shuffles or
 // shared-memory exchanges between lanes.
 //
-// What bounds it: instruction fetch and issue.  An iteration is about 12,800
-// instructions for 32 configurations, most of them straight-line code of more
-// than the instruction cache holds.  (Four lanes per configuration, with the
-// Jacobian, Gram matrix and factor in shared memory, took 16,000
-// warp-instructions per iteration for 8 configurations: 20.7 ms for 1,048,576
-// configurations, 667 us for 4,099 and 410 us for 32, against 7.2 ms, 330 us
-// and 150 us here.)  Layout:
+// What bounds it: instruction fetch and dependent latency.  An iteration is
+// about 11,000 instructions for 32 configurations, most of them straight-line
+// code of more than the instruction cache holds; a scheduler has two warps.
+// (Four lanes per configuration, with the Jacobian, Gram matrix and factor in
+// shared memory, took 16,000 warp-instructions per iteration for 8
+// configurations: 20.7 ms for 1,048,576 configurations, 667 us for 4,099 and
+// 410 us for 32, against 6.2 ms, 270 us and 140 us here.)  Layout:
 //   * shared memory per configuration: 129 float2 (TREE_PAIRS), lane-major
 //     (pair e of lane l at [e * 32 + l]: conflict-free 64-bit accesses at
 //     immediate offsets); seven warps of 32 configurations fill an SM's 227 KB;
-//   * the two legs, and the two arms, run the same code in a loop over the
-//     side (half the instruction footprint);
+//   * the left and the right leg, and the two arms, go through FK, Jacobian,
+//     Gram and solve together, two values per instruction (mcp_pack.cuh; with
+//     the limbs one after the other 7.2 ms instead of 6.5 ms);
+//   * Jacobian segments are built in loops over a limb's joints that fit the
+//     scheduler's own instruction buffer;
 //   * warps go through an iteration in step: a barrier between its phases
-//     (TREE_SYNCS of them) keeps them within the same few KB of code, so that
-//     one fetch serves several.  Without barriers the warps fetch seven places
-//     at once: 13.0 ms instead of 8.5 ms for 1,048,576;
+//     (TREE_SYNCS of them after the stopping test) keeps them within the same
+//     few KB of code, so that one fetch serves several.  Without barriers the
+//     warps fetched seven places at once: 13.0 ms instead of 8.5 ms;
 //   * in two teams, of the first TREE_TEAM warps and the rest (one warp of each
-//     on a scheduler): a team takes its FP64 acceptances together, when one of
-//     its warps has 32 configurations waiting (those with at least
-//     TREE_ACCEPT_MIN take part), while the other team steps on in FP32.  Up to
-//     96 configurations wait per warp, and a token lets one team at a time
-//     accept: the teams settle in opposite phases instead of sharing the FP64
-//     unit and then leaving it idle together (8.5 -> 7.2 ms for 1,048,576);
+//     on a scheduler): a team takes its FP64 acceptances together, when each of
+//     its warps has 32 configurations waiting, while the other team steps on in
+//     FP32.  Up to 96 configurations wait per warp, and a token lets one team
+//     at a time accept: the teams settle in opposite phases instead of sharing
+//     the FP64 unit and then leaving it idle together (8.5 -> 7.2 ms);
+//   * the next chunk of starts is claimed while the last is used up, and
+//     prefetched (the refill 6,000 -> 3,000 cycles of an iteration of 65,000);
 //   * the floating base's prismatic joints have constant Jacobian columns:
 //     these, and their share of the Gram matrix, are kernel parameters.
 //
@@ -37,6 +41,7 @@
 #pragma once
 
 #include "mcp_group.cuh"
+#include "mcp_pack.cuh"
 
 namespace mcp {
 
@@ -46,11 +51,12 @@ namespace mcp {
 constexpr int TR_LEG = 6, TR_ARM = 7;
 constexpr int TR_LEG0 = 6, TR_WAIST = 18, TR_TORSO = 19, TR_NECK = 20, TR_ARM0 = 22;
 
-// float2 slots of one configuration's shared memory
-constexpr int TP_LIMB = 0;                                  // per limb joint: 6-row segment (3), CoM (1)
-constexpr int TP_ARM = TP_LIMB + 4 * 2 * TR_LEG;            // legs first, then arms
-constexpr int TP_BASE = TP_ARM + 4 * 2 * TR_ARM;            // per revolute base joint: left foot (3), right foot (3), CoM (1)
-constexpr int TP_UP = TP_BASE + 7 * 3;                      // waist, torso, neck joints: CoM
+// float2 slots of one configuration's shared memory; in a limb's slots x is
+// the left limb's value, y the right limb's
+constexpr int TP_LEG = 0;                        // per leg joint: axis and origin, then the 6-row segment (6), CoM (2)
+constexpr int TP_ARM = TP_LEG + 8 * TR_LEG;      // per arm joint: the same
+constexpr int TP_BASE = TP_ARM + 8 * TR_ARM;     // per revolute base joint: the feet's segments (6), CoM (1: x, y rows)
+constexpr int TP_UP = TP_BASE + 7 * 3;           // waist, torso, neck joints: CoM (x, y rows)
 constexpr int TREE_PAIRS = TP_UP + 4;
 
 template <class P>
@@ -100,18 +106,30 @@ __host__ __device__ constexpr int tree_part(int j) {
   return base[j];
 }
 
-// Constants of the prismatic base chain (see GrpTables) and what follows from them.
+// Constants of the prismatic base chain (see GrpTables) and what follows from
+// them, and the limbs' model data in left / right pairs.
+template <int N>
+struct TreeLimb {
+  float2 t[N][3];    // offset's translation
+  float2 com[N][3];
+  float2 mass[N];
+  float2 nmsub[N];   // minus the subtree mass
+  float2 ft[3];      // task frame's translation
+};
 template <class P>
 struct TreeConst {
+  TreeLimb<TR_LEG> leg;
+  TreeLimb<TR_ARM> arm;
+  float2 Pr[9], Pp[3], Qr[9], Qp[3];  // the feet's error frames: P^-1, Q^-1
+  float2 jt[3][3];     // translational rows of the feet's Jacobian columns of the prismatic joints,
+  float2 LL[6];        // their share of J J^T: the feet's diagonal blocks (lower 3 x 3),
+  float2 CL[6];        // CoM against each foot,
+  float LR[9];         // right foot against left foot
+  float jc[3][2];      // CoM rows of their columns
   float R[9];          // rotation after the chain
   float a[3][3];       // joint axes
   float c[3][3];       // origins at q = 0
   float mc[3][3];      // m_i R_i com_i
-  float jt[2][3][3];   // translational rows of the feet's Jacobian columns
-  float jc[3][2];      // CoM rows of their columns
-  float LL[2][6];      // their share of J J^T: the feet's diagonal blocks (lower 3 x 3),
-  float LR[9];         // right foot against left foot,
-  float CL[2][6];      // CoM against each foot
 };
 
 template <class P>
@@ -140,10 +158,33 @@ struct TreeArgs {
 };
 
 // Host: the constants, with the operations the kernel would use on them.
+template <int N>
+void fill_limb(const ModelT<float> &m, int jl, int jr, int fl, int fr, TreeLimb<N> &t) {
+  for (int i = 0; i < N; ++i) {
+    for (int k = 0; k < 3; ++k) {
+      t.t[i][k] = make_float2(m.X[jl + i][4 * k + 3], m.X[jr + i][4 * k + 3]);
+      t.com[i][k] = make_float2(m.com[jl + i][k], m.com[jr + i][k]);
+    }
+    t.mass[i] = make_float2(m.mass[jl + i], m.mass[jr + i]);
+    t.nmsub[i] = make_float2(-m.msub[jl + i], -m.msub[jr + i]);
+  }
+  for (int k = 0; k < 3; ++k) t.ft[k] = make_float2(m.fX[fl][4 * k + 3], m.fX[fr][4 * k + 3]);
+}
 template <class P>
 TreeConst<P> make_tree_const(const ModelT<float> &m, const ModelT<double> &m64) {
   const GrpTables<P> g = make_grp_tables<P>(m, m64);
   TreeConst<P> t{};
+  fill_limb(m, TR_LEG0, TR_LEG0 + TR_LEG, 0, 1, t.leg);
+  fill_limb(m, TR_ARM0, TR_ARM0 + TR_ARM, 2, 3, t.arm);
+  for (int r = 0; r < 3; ++r) {
+    for (int c = 0; c < 3; ++c) {
+      t.Pr[3 * r + c] = make_float2(m.cPinv[0][4 * r + c], m.cPinv[1][4 * r + c]);
+      t.Qr[3 * r + c] = make_float2(m.cQinv[0][4 * r + c], m.cQinv[1][4 * r + c]);
+    }
+    t.Pp[r] = make_float2(m.cPinv[0][4 * r + 3], m.cPinv[1][4 * r + 3]);
+    t.Qp[r] = make_float2(m.cQinv[0][4 * r + 3], m.cQinv[1][4 * r + 3]);
+  }
+  float jt[2][3][3], LL[2][6] = {}, CL[2][6] = {};
   for (int e = 0; e < 9; ++e) t.R[e] = g.pre_R[2][e];
   for (int i = 0; i < 3; ++i) {
     for (int r = 0; r < 3; ++r) {
@@ -158,18 +199,22 @@ TreeConst<P> make_tree_const(const ModelT<float> &m, const ModelT<double> &m64) 
       for (int r = 0; r < 3; ++r) {
         const float *Pi = m.cPinv[s] + 4 * r;
         const float p2 = Pi[2] * t.a[i][2];
-        t.jt[s][i][r] = std::fmaf(Pi[0], t.a[i][0], std::fmaf(Pi[1], t.a[i][1], p2));
+        jt[s][i][r] = std::fmaf(Pi[0], t.a[i][0], std::fmaf(Pi[1], t.a[i][1], p2));
       }
-  }
-  for (int i = 0; i < 3; ++i) {
-    for (int r = 0; r < 3; ++r)
-      for (int c = 0; c < 3; ++c) t.LR[3 * r + c] = std::fmaf(t.jt[1][i][r], t.jt[0][i][c], t.LR[3 * r + c]);
+    for (int r = 0; r < 3; ++r) {
+      t.jt[i][r] = make_float2(jt[0][i][r], jt[1][i][r]);
+      for (int c = 0; c < 3; ++c) t.LR[3 * r + c] = std::fmaf(jt[1][i][r], jt[0][i][c], t.LR[3 * r + c]);
+    }
     for (int s = 0; s < 2; ++s) {
       for (int r = 0; r < 3; ++r)
-        for (int c = 0; c <= r; ++c) t.LL[s][tri(r, c)] = std::fmaf(t.jt[s][i][r], t.jt[s][i][c], t.LL[s][tri(r, c)]);
+        for (int c = 0; c <= r; ++c) LL[s][tri(r, c)] = std::fmaf(jt[s][i][r], jt[s][i][c], LL[s][tri(r, c)]);
       for (int r = 0; r < 2; ++r)
-        for (int c = 0; c < 3; ++c) t.CL[s][3 * r + c] = std::fmaf(t.jc[i][r], t.jt[s][i][c], t.CL[s][3 * r + c]);
+        for (int c = 0; c < 3; ++c) CL[s][3 * r + c] = std::fmaf(t.jc[i][r], jt[s][i][c], CL[s][3 * r + c]);
     }
+  }
+  for (int e = 0; e < 6; ++e) {
+    t.LL[e] = make_float2(LL[0][e], LL[1][e]);
+    t.CL[e] = make_float2(CL[0][e], CL[1][e]);
   }
   return t;
 }
@@ -242,40 +287,94 @@ __device__ __forceinline__ float2 tree_com_col(V3<float> z, V3<float> o, V3<floa
   return make_float2(__fmul_rn(d.x, inv_mass), __fmul_rn(d.y, inv_mass));
 }
 
-// What the Jacobian of a pose-like constraint needs from its residual.
-struct TreePose {
-  V3<float> x, phi;
-  float beta;
-};
-// Log map, stored residual rows and squared norm of a pose-like constraint.
-__device__ __forceinline__ float tree_pose_tail(const float (&Rerr)[9], V3<float> t, TreePose &e, float (&F)[6]) {
-  const auto lg = so3_log<OpsF32, float>(Rerr);
-  e.phi = lg.phi;
-  e.beta = jl_inv_beta<float>(lg.theta, lg.s, lg.c);
-  F[0] = t.x;
-  F[1] = t.y;
-  F[2] = t.z;
-  F[3] = lg.phi.x;
-  F[4] = lg.phi.y;
-  F[5] = lg.phi.z;
-  return fmaf(t.x, t.x, fmaf(t.y, t.y, fmaf(t.z, t.z, fmaf(lg.phi.x, lg.phi.x, fmaf(lg.phi.y, lg.phi.y, lg.phi.z * lg.phi.z)))));
-}
-// 6-row segment of a revolute joint with axis z and origin o
-__device__ __forceinline__ void tree_seg6(const float (&G)[9], const TreePose &e, V3<float> z, V3<float> o, float2 (&v)[3]) {
-  const V3<float> vt = mulv(G, cross(z, sub(e.x, o)));
-  const V3<float> w = jl_inv_apply(e.phi, e.beta, mulv(G, z));
-  v[0] = make_float2(vt.x, vt.y);
-  v[1] = make_float2(vt.z, w.x);
-  v[2] = make_float2(w.y, w.z);
-}
-__device__ __forceinline__ void unpack6(const float2 (&v)[3], float (&f)[6]) {
+// The same for a left and a right joint of one structure: offset translation
+// t, task-frame translation ft, masses and CoM offsets in pairs.
+template <int CODE, int TM>
+__device__ __forceinline__ void tree_joint2(float2 (&T)[12], const float2 *t, float2 q) {
+  constexpr int p0 = xr_perm(CODE, 0), p1 = xr_perm(CODE, 1), p2 = xr_perm(CODE, 2);
+  float2 sn, cs;
+  sincos2_f32(q, sn, cs);
+  const float2 nsn = neg2(sn);
+  const float2 csa = xr_neg(CODE, 0) ? neg2(cs) : cs, sna = xr_neg(CODE, 0) ? sn : nsn;  // sna = -(sign sn)
+  const float2 csb = xr_neg(CODE, 1) ? neg2(cs) : cs, snb = xr_neg(CODE, 1) ? nsn : sn;
 #pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    f[2 * i] = v[i].x;
-    f[2 * i + 1] = v[i].y;
+  for (int r = 0; r < 3; ++r) {
+    float2 p = T[4 * r + 3];
+    if constexpr (TM & 4) p = __ffma2_rn(T[4 * r + 2], t[2], p);
+    if constexpr (TM & 2) p = __ffma2_rn(T[4 * r + 1], t[1], p);
+    if constexpr (TM & 1) p = __ffma2_rn(T[4 * r], t[0], p);
+    const float2 a = T[4 * r + p0], b = T[4 * r + p1], c = T[4 * r + p2];
+    if constexpr (p0 < p1) {
+      T[4 * r] = __ffma2_rn(csa, a, __fmul2_rn(snb, b));
+      T[4 * r + 1] = __ffma2_rn(sna, a, __fmul2_rn(csb, b));
+    } else {
+      T[4 * r] = __ffma2_rn(snb, b, __fmul2_rn(csa, a));
+      T[4 * r + 1] = __ffma2_rn(csb, b, __fmul2_rn(sna, a));
+    }
+    T[4 * r + 2] = xr_neg(CODE, 2) ? neg2(c) : c;
+    T[4 * r + 3] = p;
   }
 }
-
+template <int CODE, int TM>
+__device__ __forceinline__ void tree_frame2(const float2 (&T)[12], const float2 *ft, float2 (&R)[9], V3p &p) {
+  float2 o[3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const float2 v = T[4 * r + xr_perm(CODE, c)];
+      R[3 * r + c] = xr_neg(CODE, c) ? neg2(v) : v;
+    }
+    float2 v = T[4 * r + 3];
+    if constexpr (TM & 4) v = __ffma2_rn(T[4 * r + 2], ft[2], v);
+    if constexpr (TM & 2) v = __ffma2_rn(T[4 * r + 1], ft[1], v);
+    if constexpr (TM & 1) v = __ffma2_rn(T[4 * r], ft[0], v);
+    o[r] = v;
+  }
+  p = V3p{o[0], o[1], o[2]};
+}
+__device__ __forceinline__ V3p load_axis(const float2 *s) { return V3p{s[0], s[32], s[64]}; }
+__device__ __forceinline__ V3p load_origin(const float2 *s) { return V3p{s[96], s[128], s[160]}; }
+// FK of a pair of limbs of N joints (the first joint's class index J0), from
+// the frame T of their parent: axes and origins into the joints' slots (read
+// back for the CoM columns: kept in registers they would spill), the CoM
+// columns after them; returns the limbs' subtree moments, T the tip's frame.
+template <class P, int J0, int N>
+__device__ __forceinline__ V3p tree_limbs(const TreeLimb<N> &m, float2 (&T)[12], const float (&q)[P::D], float inv_mass,
+                                          float2 *__restrict__ slot) {
+  V3p C[N];
+  static_for<N>([&](auto II) {
+    constexpr int i = decltype(II)::value, j = J0 + i;
+    tree_joint2<P::xrot(j), P::xtmask(j)>(T, m.t[i], make_float2(q[j], q[j + N]));
+    float2 v[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+      v[r] = __fmul2_rn(m.mass[i], __ffma2_rn(T[4 * r], m.com[i][0],
+                                              __ffma2_rn(T[4 * r + 1], m.com[i][1],
+                                                         __ffma2_rn(T[4 * r + 2], m.com[i][2], T[4 * r + 3]))));
+    C[i] = V3p{v[0], v[1], v[2]};
+    float2 *s = slot + 8 * 32 * i;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      s[r * 32] = T[4 * r + 2];
+      s[(3 + r) * 32] = T[4 * r + 3];
+    }
+  });
+  static_for<N>([&](auto II) {
+    constexpr int i = N - 1 - decltype(II)::value;
+    if constexpr (i + 1 < N)
+      C[i] = V3p{add2_apart(C[i].x, C[i + 1].x), add2_apart(C[i].y, C[i + 1].y), add2_apart(C[i].z, C[i + 1].z)};
+    // (1/M) z x (C - M_j o), x and y
+    const float2 nM = m.nmsub[i];
+    const V3p z = load_axis(slot + 8 * 32 * i), o = load_origin(slot + 8 * 32 * i);
+    const V3p rr{__ffma2_rn(nM, o.x, C[i].x), __ffma2_rn(nM, o.y, C[i].y), __ffma2_rn(nM, o.z, C[i].z)};
+    const float2 dx = __ffma2_rn(z.y, rr.z, __fmul2_rn(neg2(z.z), rr.y));
+    const float2 dy = __ffma2_rn(z.z, rr.x, __fmul2_rn(neg2(z.x), rr.z));
+    slot[(8 * i + 6) * 32] = __fmul2_rn(dx, both(inv_mass));
+    slot[(8 * i + 7) * 32] = __fmul2_rn(dy, both(inv_mass));
+  });
+  return C[0];
+}
 // Warps of a block that go through the iterations in step with one another.
 struct TreeTeam {
   int id, threads;  // named barrier and the number of threads that meet at it
@@ -309,23 +408,25 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
   const auto at = [&](int e) -> float2 & { return sm[e * 32]; };
   const float inv_mass = m.inv_mass;
 
+  float qv[P::D];  // loaded together: one latency, not one per chain
+#pragma unroll
+  for (int j = 0; j < P::D; ++j) qv[j] = q[j];
   float F[K];
-  float r2f[2] = {0.f, 0.f};           // squared residual norms of the feet
-  V3<float> zb[3], ob[3], mb[3];       // revolute base joints: axis, origin, moment
+  V3<float> mb[3];                     // revolute base joints: moments
   V3<float> zw[2], ow[2], mw[2];       // waist and torso
   V3<float> Cneck;                     // subtree moments of the torso's and pelvis's children
-  V3<float> Cleg[2], Carm[2];
+  V3p Cleg, Carm;
   float px[3][2];                      // prismatic joints: moments, x and y
-  float T5[12], T19[12];
+  float T5[12], T19[12];               // pelvis and torso frames
   // trunk and neck
   {
     float T[12];
     float o0 = 0.f, o1 = 0.f, o2 = 0.f, x0 = 0.f, x1 = 0.f, x2 = 0.f;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      o0 = fmaf(q[i], a.t.a[i][0], o0);
-      o1 = fmaf(q[i], a.t.a[i][1], o1);
-      o2 = fmaf(q[i], a.t.a[i][2], o2);
+      o0 = fmaf(qv[i], a.t.a[i][0], o0);
+      o1 = fmaf(qv[i], a.t.a[i][1], o1);
+      o2 = fmaf(qv[i], a.t.a[i][2], o2);
       x0 = __fadd_rn(a.t.c[i][0], o0);
       x1 = __fadd_rn(a.t.c[i][1], o1);
       x2 = __fadd_rn(a.t.c[i][2], o2);
@@ -341,16 +442,19 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
     T[11] = x2;
     static_for<3>([&](auto II) {
       constexpr int i = decltype(II)::value, j = 3 + i;
-      tree_joint<P::xrot(j), P::xtmask(j)>(T, m.X[j], q[j]);
-      zb[i] = V3<float>{T[2], T[6], T[10]};
-      ob[i] = V3<float>{T[3], T[7], T[11]};
+      tree_joint<P::xrot(j), P::xtmask(j)>(T, m.X[j], qv[j]);
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {  // the same for both feet
+        at(TP_BASE + 7 * i + r) = both(T[4 * r + 2]);
+        at(TP_BASE + 7 * i + 3 + r) = both(T[4 * r + 3]);
+      }
       mb[i] = tree_moment(T, m.com[j], m.mass[j]);
     });
 #pragma unroll
     for (int e = 0; e < 12; ++e) T5[e] = T[e];
     static_for<2>([&](auto II) {
       constexpr int i = decltype(II)::value, j = TR_WAIST + i;
-      tree_joint<P::xrot(j), P::xtmask(j)>(T, m.X[j], q[j]);
+      tree_joint<P::xrot(j), P::xtmask(j)>(T, m.X[j], qv[j]);
       zw[i] = V3<float>{T[2], T[6], T[10]};
       ow[i] = V3<float>{T[3], T[7], T[11]};
       mw[i] = tree_moment(T, m.com[j], m.mass[j]);
@@ -360,7 +464,7 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
     V3<float> zn[2], on[2], mn[2];
     static_for<2>([&](auto II) {
       constexpr int i = decltype(II)::value, j = TR_NECK + i;
-      tree_joint<P::xrot(j), P::xtmask(j)>(T, m.X[j], q[j]);
+      tree_joint<P::xrot(j), P::xtmask(j)>(T, m.X[j], qv[j]);
       zn[i] = V3<float>{T[2], T[6], T[10]};
       on[i] = V3<float>{T[3], T[7], T[11]};
       mn[i] = tree_moment(T, m.com[j], m.mass[j]);
@@ -369,139 +473,109 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
     Cneck = tree_add(mn[0], mn[1]);
     at(TP_UP + 2) = tree_com_col(zn[0], on[0], Cneck, m.msub[TR_NECK], inv_mass);
   }
-  // legs: FK, CoM columns, the foot's residual and its 6-row segments
-#pragma unroll 1
-  for (int s = 0; s < 2; ++s) {
-    float T[12];
-#pragma unroll
-    for (int e = 0; e < 12; ++e) T[e] = T5[e];
-    V3<float> z[TR_LEG], o[TR_LEG], C[TR_LEG];
-    const int j0 = TR_LEG0 + s * TR_LEG;
-    static_for<TR_LEG>([&](auto II) {
-      constexpr int i = decltype(II)::value, jr = TR_LEG0 + i;
-      tree_joint<P::xrot(jr), P::xtmask(jr)>(T, m.X[j0 + i], q[j0 + i]);
-      z[i] = V3<float>{T[2], T[6], T[10]};
-      o[i] = V3<float>{T[3], T[7], T[11]};
-      C[i] = tree_moment(T, m.com[j0 + i], m.mass[j0 + i]);
-    });
-    float2 *leg = sm + (TP_LIMB + 4 * TR_LEG * s) * 32;
-    static_for<TR_LEG>([&](auto II) {
-      constexpr int i = TR_LEG - 1 - decltype(II)::value;
-      if constexpr (i + 1 < TR_LEG) C[i] = tree_add(C[i], C[i + 1]);
-      leg[(4 * i + 3) * 32] = tree_com_col(z[i], o[i], C[i], m.msub[j0 + i], inv_mass);
-    });
-    float Ra[9], Pr[9], Qr[9], RaQ[9], Rerr[9], f6[6];
-    V3<float> pa;
-    tree_frame<P::frot(0), P::ftmask(0)>(T, m.fX[s], Ra, pa);
-    load_R(m.cPinv[s], Pr);
-    load_R(m.cQinv[s], Qr);
-    const V3<float> Pp = load_p(m.cPinv[s]);
-    TreePose e;
-    mul33(Ra, Qr, RaQ);
-    mul33(Pr, RaQ, Rerr);
-    e.x = add_rot_t<7>(pa, Ra, load_p(m.cQinv[s]));
-    const V3<float> tx = mulv(Pr, e.x);
-    const float n2 =
-        tree_pose_tail(Rerr, V3<float>{__fadd_rn(tx.x, Pp.x), __fadd_rn(tx.y, Pp.y), __fadd_rn(tx.z, Pp.z)}, e, f6);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      float2 v[3];
-      tree_seg6(Pr, e, zb[i], ob[i], v);
-      float2 *b = sm + (TP_BASE + 7 * i + 3 * s) * 32;
-#pragma unroll
-      for (int r = 0; r < 3; ++r) b[r * 32] = v[r];
-    }
-#pragma unroll
-    for (int i = 0; i < TR_LEG; ++i) {
-      float2 v[3];
-      tree_seg6(Pr, e, z[i], o[i], v);
-#pragma unroll
-      for (int r = 0; r < 3; ++r) leg[(4 * i + r) * 32] = v[r];
-    }
-    if (s == 0) {
-      r2f[0] = n2;
-      Cleg[0] = C[0];
-#pragma unroll
-      for (int i = 0; i < 6; ++i) F[i] = f6[i];
-    } else {
-      r2f[1] = n2;
-      Cleg[1] = C[0];
-#pragma unroll
-      for (int i = 0; i < 6; ++i) F[6 + i] = f6[i];
-    }
-  }
-  team.sync();
-  // arms: FK, CoM columns, axes and origins into the segments' slots
-  float Ra[9], Rb[9];
-  V3<float> pa, pb{0.f, 0.f, 0.f};
-#pragma unroll
-  for (int i = 0; i < 9; ++i) Rb[i] = 0.f;
-#pragma unroll 1
-  for (int s = 0; s < 2; ++s) {
-    float T[12];
-#pragma unroll
-    for (int e = 0; e < 12; ++e) T[e] = T19[e];
-    V3<float> z[TR_ARM], o[TR_ARM], C[TR_ARM];
-    const int j0 = TR_ARM0 + s * TR_ARM;
-    float2 *arm = sm + (TP_ARM + 4 * TR_ARM * s) * 32;
-    static_for<TR_ARM>([&](auto II) {
-      constexpr int i = decltype(II)::value, jr = TR_ARM0 + i;
-      tree_joint<P::xrot(jr), P::xtmask(jr)>(T, m.X[j0 + i], q[j0 + i]);
-      z[i] = V3<float>{T[2], T[6], T[10]};
-      o[i] = V3<float>{T[3], T[7], T[11]};
-      C[i] = tree_moment(T, m.com[j0 + i], m.mass[j0 + i]);
-      arm[(4 * i) * 32] = make_float2(z[i].x, z[i].y);
-      arm[(4 * i + 1) * 32] = make_float2(z[i].z, o[i].x);
-      arm[(4 * i + 2) * 32] = make_float2(o[i].y, o[i].z);
-    });
-    static_for<TR_ARM>([&](auto II) {
-      constexpr int i = TR_ARM - 1 - decltype(II)::value;
-      if constexpr (i + 1 < TR_ARM) C[i] = tree_add(C[i], C[i + 1]);
-      arm[(4 * i + 3) * 32] = tree_com_col(z[i], o[i], C[i], m.msub[j0 + i], inv_mass);
-    });
-#pragma unroll
-    for (int i = 0; i < 9; ++i) Ra[i] = Rb[i];
-    pa = pb;
-    tree_frame<P::frot(2), P::ftmask(2)>(T, m.fX[2 + s], Rb, pb);
-    if (s == 0) Carm[0] = C[0];
-    else Carm[1] = C[0];
-  }
-  team.sync();
-  // the hands' relative pose: G = P^-1_R R_a^T, R_err = G R_b, t = G (p_b - p_a) + P^-1_p
-  float G[9];
-  TreePose eh;
-  float r2h;
+  // legs and arms, left and right together
+  float2 Rf[9], Rh[9];
+  V3p pf, ph;
   {
-    float Pr[9], RaT[9], Rerr[9], f6[6];
+    float2 T[12];
+#pragma unroll
+    for (int e = 0; e < 12; ++e) T[e] = both(T5[e]);
+    Cleg = tree_limbs<P, TR_LEG0, TR_LEG>(a.t.leg, T, qv, inv_mass, sm + TP_LEG * 32);
+    tree_frame2<P::frot(0), P::ftmask(0)>(T, a.t.leg.ft, Rf, pf);
+  }
+  team.sync();
+  {
+    float2 T[12];
+#pragma unroll
+    for (int e = 0; e < 12; ++e) T[e] = both(T19[e]);
+    Carm = tree_limbs<P, TR_ARM0, TR_ARM>(a.t.arm, T, qv, inv_mass, sm + TP_ARM * 32);
+    tree_frame2<P::frot(2), P::ftmask(2)>(T, a.t.arm.ft, Rh, ph);
+  }
+  team.sync();
+  // error rotations and translations: the feet, R_err = P^-1_R R_a Q^-1_R,
+  // t = P^-1_R x + P^-1_p at x = p_a + R_a Q^-1_p; the hands, G = P^-1_R R_a^T,
+  // R_err = G R_b, t = G (p_b - p_a) + P^-1_p
+  float2 Ef[9], tf[3];
+  float G[9], Eh[9], th[3];
+  PosePair ef;
+  {
+    float2 RaQ[9];
+    mul33_2(Rf, a.t.Qr, RaQ);
+    mul33_2(a.t.Pr, RaQ, Ef);
+    ef.x = pf;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      ef.x = V3p{__ffma2_rn(Rf[k], a.t.Qp[k], ef.x.x), __ffma2_rn(Rf[3 + k], a.t.Qp[k], ef.x.y),
+                 __ffma2_rn(Rf[6 + k], a.t.Qp[k], ef.x.z)};
+#pragma unroll
+    for (int r = 0; r < 3; ++r) tf[r] = __fadd2_rn(row2(a.t.Pr + 3 * r, ef.x), a.t.Pp[r]);
+    float Pr[9], RaT[9], Rb[9];
     load_R(m.cPinv[2], Pr);
     const V3<float> Pp = load_p(m.cPinv[2]);
 #pragma unroll
     for (int r = 0; r < 3; ++r)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) RaT[3 * r + c] = Ra[3 * c + r];
+      for (int c = 0; c < 3; ++c) {
+        RaT[3 * r + c] = Rh[3 * c + r].x;
+        Rb[3 * r + c] = Rh[3 * r + c].y;
+      }
     mul33(Pr, RaT, G);
-    mul33(G, Rb, Rerr);
-    const V3<float> tx = mulv(G, sub(pb, pa));
-    eh.x = pb;
-    r2h = tree_pose_tail(Rerr, V3<float>{__fadd_rn(tx.x, Pp.x), __fadd_rn(tx.y, Pp.y), __fadd_rn(tx.z, Pp.z)}, eh, f6);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) F[12 + i] = f6[i];
+    mul33(G, Rb, Eh);
+    const V3<float> tx = mulv(G, V3<float>{ph.x.y - ph.x.x, ph.y.y - ph.y.x, ph.z.y - ph.z.x});
+    th[0] = __fadd_rn(tx.x, Pp.x);
+    th[1] = __fadd_rn(tx.y, Pp.y);
+    th[2] = __fadd_rn(tx.z, Pp.z);
   }
+  // log maps: left foot, right foot, hands, one copy of the code
+  float n2[3];
+  V3<float> phi[3];
+  float beta[3];
+#pragma unroll 1
+  for (int s = 0; s < 3; ++s) {
+    float E[9], t[3];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) E[i] = s == 0 ? Ef[i].x : (s == 1 ? Ef[i].y : Eh[i]);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) t[i] = s == 0 ? tf[i].x : (s == 1 ? tf[i].y : th[i]);
+    const auto lg = so3_log<OpsF32, float>(E);
+    const float be = jl_inv_beta<float>(lg.theta, lg.s, lg.c);
+    const float f[6] = {t[0], t[1], t[2], lg.phi.x, lg.phi.y, lg.phi.z};
+    const float n = fmaf(f[0], f[0], fmaf(f[1], f[1], fmaf(f[2], f[2], fmaf(f[3], f[3], fmaf(f[4], f[4], f[5] * f[5])))));
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+      if (s == u) {
+        n2[u] = n;
+        phi[u] = lg.phi;
+        beta[u] = be;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) F[6 * u + i] = f[i];
+      }
+  }
+  ef.phi = V3p{make_float2(phi[0].x, phi[1].x), make_float2(phi[0].y, phi[1].y), make_float2(phi[0].z, phi[1].z)};
+  ef.nphi = neg2(ef.phi);
+  ef.beta = make_float2(beta[0], beta[1]);
   // trunk moments and CoM columns, the CoM residual
   float r2c;
   [[maybe_unused]] int hmode = 2;
   [[maybe_unused]] float hn0 = 0.f, hn1 = 0.f;
   {
-    V3<float> C = tree_add(tree_add(tree_add(mw[1], Cneck), Carm[0]), Carm[1]);
+    const auto base_com = [&](int i, V3<float> C) {
+      const float2 *b = sm + (TP_BASE + 7 * i) * 32;
+      return tree_com_col(V3<float>{b[0].x, b[32].x, b[64].x}, V3<float>{b[96].x, b[128].x, b[160].x}, C, m.msub[3 + i],
+                          inv_mass);
+    };
+    V3<float> C = tree_add(tree_add(tree_add(mw[1], Cneck), V3<float>{Carm.x.x, Carm.y.x, Carm.z.x}),
+                           V3<float>{Carm.x.y, Carm.y.y, Carm.z.y});
     at(TP_UP + 1) = tree_com_col(zw[1], ow[1], C, m.msub[TR_TORSO], inv_mass);
     C = tree_add(mw[0], C);
     at(TP_UP) = tree_com_col(zw[0], ow[0], C, m.msub[TR_WAIST], inv_mass);
-    C = tree_add(tree_add(tree_add(mb[2], Cleg[0]), Cleg[1]), C);
-    at(TP_BASE + 7 * 2 + 6) = tree_com_col(zb[2], ob[2], C, m.msub[5], inv_mass);
+    C = tree_add(tree_add(tree_add(mb[2], V3<float>{Cleg.x.x, Cleg.y.x, Cleg.z.x}),
+                          V3<float>{Cleg.x.y, Cleg.y.y, Cleg.z.y}), C);
+    at(TP_BASE + 7 * 2 + 6) = base_com(2, C);
     C = tree_add(mb[1], C);
-    at(TP_BASE + 7 * 1 + 6) = tree_com_col(zb[1], ob[1], C, m.msub[4], inv_mass);
+    at(TP_BASE + 7 * 1 + 6) = base_com(1, C);
     C = tree_add(mb[0], C);
-    at(TP_BASE + 6) = tree_com_col(zb[0], ob[0], C, m.msub[3], inv_mass);
+    at(TP_BASE + 6) = base_com(0, C);
     const float t0 = __fadd_rn(px[0][0], __fadd_rn(px[1][0], __fadd_rn(px[2][0], C.x)));
     const float t1 = __fadd_rn(px[0][1], __fadd_rn(px[1][1], __fadd_rn(px[2][1], C.y)));
     float f0, f1;
@@ -519,7 +593,7 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
     F[19] = f1;
     r2c = fmaf(f0, f0, __fmul_rn(f1, f1));
   }
-  const float r2 = __fadd_rn(__fadd_rn(r2f[0], r2f[1]), __fadd_rn(r2h, r2c));
+  const float r2 = __fadd_rn(__fadd_rn(n2[0], n2[1]), __fadd_rn(n2[2], r2c));
   bool done = false;
   if (act) {
     if (!(r2 <= FLT_MAX)) {
@@ -553,42 +627,75 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
       jc[i] = fold(jc[i]);
       at(TP_BASE + 7 * i + 6) = fold(at(TP_BASE + 7 * i + 6));
     }
-#pragma unroll 2
-    for (int l = 0; l < 2 * (TR_LEG + TR_ARM); ++l) at(TP_LIMB + 4 * l + 3) = fold(at(TP_LIMB + 4 * l + 3));
+#pragma unroll 1
+    for (int l = 0; l < TR_LEG + TR_ARM; ++l) {
+      const float2 gx = at(TP_LEG + 8 * l + 6), gy = at(TP_LEG + 8 * l + 7);
+      const float2 u = fold(make_float2(gx.x, gy.x)), w = fold(make_float2(gx.y, gy.y));
+      at(TP_LEG + 8 * l + 6) = make_float2(u.x, w.x);
+      at(TP_LEG + 8 * l + 7) = make_float2(u.y, w.y);
+    }
 #pragma unroll
     for (int i = 0; i < 4; ++i) at(TP_UP + i) = fold(at(TP_UP + i));
   }
   // Gram matrix (then its factor) in packed lower-triangular form; only the
   // structural nonzeros are touched
   float L[K * (K + 1) / 2];
+  float2 ca[3], cl[3];  // CoM block: partial sums of the arms and of the legs
+#pragma unroll
+  for (int i = 0; i < 3; ++i) ca[i] = cl[i] = make_float2(0.f, 0.f);
+  const auto com_add2 = [](float2 (&p)[3], float2 gx, float2 gy) {
+    p[0] = __ffma2_rn(gx, gx, p[0]);
+    p[1] = __ffma2_rn(gy, gx, p[1]);
+    p[2] = __ffma2_rn(gy, gy, p[2]);
+  };
   // hands' block and their CoM rows, with the arms' segments built in place
+  // (joints above frame a enter with -1, above b with +1): the left arm's
+  // joints first, then the right's
   {
     float H[21], CH[12];
 #pragma unroll
     for (int i = 0; i < 21; ++i) H[i] = 0.f;
 #pragma unroll
     for (int i = 0; i < 12; ++i) CH[i] = 0.f;
-    float2 *arm = sm + TP_ARM * 32;
-#pragma unroll 1
-    for (int l = 0; l < 2 * TR_ARM; ++l, arm += 4 * 32) {
-      float2 v[3] = {arm[0], arm[32], arm[64]};
-      const float2 c = arm[96];
-      const float sg = l < TR_ARM ? -1.f : 1.f;  // joints above frame a enter with -1, above b with +1
-      tree_seg6(G, eh, V3<float>{v[0].x, v[0].y, v[1].x}, V3<float>{v[1].y, v[2].x, v[2].y}, v);
-#pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        v[r] = make_float2(sg * v[r].x, sg * v[r].y);
-        arm[r * 32] = v[r];
-      }
-      float f[6];
-      unpack6(v, f);
+    const auto add = [&](const float (&f)[6], float gx, float gy) {
 #pragma unroll
       for (int i = 0; i < 6; ++i) {
 #pragma unroll
         for (int k = 0; k <= i; ++k) H[tri(i, k)] = fmaf(f[i], f[k], H[tri(i, k)]);
-        CH[i] = fmaf(c.x, f[i], CH[i]);
-        CH[6 + i] = fmaf(c.y, f[i], CH[6 + i]);
+        CH[i] = fmaf(gx, f[i], CH[i]);
+        CH[6 + i] = fmaf(gy, f[i], CH[6 + i]);
       }
+    };
+    float2 G2[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) G2[i] = make_float2(-G[i], G[i]);
+    PosePair eh;
+    eh.x = V3p{both(ph.x.y), both(ph.y.y), both(ph.z.y)};
+    eh.phi = V3p{both(phi[2].x), both(phi[2].y), both(phi[2].z)};
+    eh.nphi = neg2(eh.phi);
+    eh.beta = both(beta[2]);
+    float2 *arm = sm + TP_ARM * 32;
+#pragma unroll 1
+    for (int l = 0; l < TR_ARM; ++l, arm += 8 * 32) {
+      float2 v[6];
+      float f[6];
+      seg6_2(G2, eh, load_axis(arm), load_origin(arm), v);
+#pragma unroll
+      for (int r = 0; r < 6; ++r) {
+        arm[r * 32] = v[r];
+        f[r] = v[r].x;
+      }
+      const float2 gx = arm[6 * 32], gy = arm[7 * 32];
+      com_add2(ca, gx, gy);
+      add(f, gx.x, gy.x);
+    }
+    arm = sm + TP_ARM * 32;
+#pragma unroll 1
+    for (int l = 0; l < TR_ARM; ++l, arm += 8 * 32) {
+      float f[6];
+#pragma unroll
+      for (int r = 0; r < 6; ++r) f[r] = arm[r * 32].y;
+      add(f, arm[6 * 32].y, arm[7 * 32].y);
     }
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
@@ -599,101 +706,108 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
     }
   }
   team.sync();
-  // feet: diagonal blocks, right against left, CoM rows
+  // feet: diagonal blocks and CoM rows (left and right together), right
+  // against left, with the segments built on the way
   {
+    float2 B[21], C[12];
 #pragma unroll
-    for (int s = 0; s < 2; ++s)
+    for (int i = 0; i < 21; ++i) B[i] = i < 6 ? a.t.LL[i < 6 ? i : 0] : make_float2(0.f, 0.f);
 #pragma unroll
-      for (int i = 0; i < 6; ++i) {
+    for (int i = 0; i < 12; ++i) {
+      const int r = i / 6, k = i % 6;
+      if (k >= 3) {
+        C[i] = make_float2(0.f, 0.f);
+      } else if constexpr (!HULL) {
+        C[i] = a.t.CL[3 * r + (k < 3 ? k : 0)];
+      } else {
+        C[i] = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int k = 0; k <= i; ++k) L[tri(6 * s + i, 6 * s + k)] = i < 3 ? a.t.LL[s][tri(i < 3 ? i : 0, i < 3 ? k : 0)] : 0.f;
-        if constexpr (!HULL) {
-          L[tri(18, 6 * s + i)] = i < 3 ? a.t.CL[s][i < 3 ? i : 0] : 0.f;
-          L[tri(19, 6 * s + i)] = i < 3 ? a.t.CL[s][3 + (i < 3 ? i : 0)] : 0.f;
-        } else {
-          float c0 = 0.f, c1 = 0.f;
-          if (i < 3) {
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-              c0 = fmaf(jc[k].x, a.t.jt[s][k][i < 3 ? i : 0], c0);
-              c1 = fmaf(jc[k].y, a.t.jt[s][k][i < 3 ? i : 0], c1);
-            }
-          }
-          L[tri(18, 6 * s + i)] = c0;
-          L[tri(19, 6 * s + i)] = c1;
-        }
+        for (int j = 0; j < 3; ++j) C[i] = __ffma2_rn(both(r == 0 ? jc[j].x : jc[j].y), a.t.jt[j][k < 3 ? k : 0], C[i]);
       }
-#pragma unroll
-    for (int i = 0; i < 6; ++i)
-#pragma unroll
-      for (int k = 0; k < 6; ++k) L[tri(6 + i, k)] = i < 3 && k < 3 ? a.t.LR[i < 3 && k < 3 ? 3 * i + k : 0] : 0.f;
-    const auto own = [&](auto SS, const float (&f)[6], float2 c) {  // a foot's block and CoM rows
-      constexpr int r0 = 6 * decltype(SS)::value;
+    }
+    const auto add = [&](const float2 (&f)[6], float2 gx, float2 gy) {
 #pragma unroll
       for (int i = 0; i < 6; ++i) {
 #pragma unroll
-        for (int k = 0; k <= i; ++k) L[tri(r0 + i, r0 + k)] = fmaf(f[i], f[k], L[tri(r0 + i, r0 + k)]);
-        L[tri(18, r0 + i)] = fmaf(c.x, f[i], L[tri(18, r0 + i)]);
-        L[tri(19, r0 + i)] = fmaf(c.y, f[i], L[tri(19, r0 + i)]);
+        for (int k = 0; k <= i; ++k) B[tri(i, k)] = __ffma2_rn(f[i], f[k], B[tri(i, k)]);
+        C[i] = __ffma2_rn(gx, f[i], C[i]);
+        C[6 + i] = __ffma2_rn(gy, f[i], C[6 + i]);
       }
     };
+    float2 Pr[9];
 #pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      float2 v[3];
-      float fl6[6], fr6[6];
+    for (int i = 0; i < 9; ++i) Pr[i] = a.t.Pr[i];
+    // the base's joints, then the legs', in one loop body
+#pragma unroll 1
+    for (int l = 0; l < 3 + TR_LEG; ++l) {
+      float2 *s = sm + (l < 3 ? TP_BASE + 7 * l : TP_LEG + 8 * (l - 3)) * 32;
+      float2 v[6];
+      seg6_2(Pr, ef, load_axis(s), load_origin(s), v);
 #pragma unroll
-      for (int r = 0; r < 3; ++r) v[r] = at(TP_BASE + 7 * b + r);
-      unpack6(v, fl6);
-#pragma unroll
-      for (int r = 0; r < 3; ++r) v[r] = at(TP_BASE + 7 * b + 3 + r);
-      unpack6(v, fr6);
-      const float2 c = at(TP_BASE + 7 * b + 6);
-      own(std::integral_constant<int, 0>{}, fl6, c);
-      own(std::integral_constant<int, 1>{}, fr6, c);
-#pragma unroll
-      for (int i = 0; i < 6; ++i)
-#pragma unroll
-        for (int k = 0; k < 6; ++k) L[tri(6 + i, k)] = fmaf(fr6[i], fl6[k], L[tri(6 + i, k)]);
-    }
-    static_for<2>([&](auto SS) {
-      constexpr int s = decltype(SS)::value;
-#pragma unroll
-      for (int i = 0; i < TR_LEG; ++i) {
-        const int e = TP_LIMB + 4 * (TR_LEG * s + i);
-        const float2 v[3] = {at(e), at(e + 1), at(e + 2)};
-        float f[6];
-        unpack6(v, f);
-        own(SS, f, at(e + 3));
+      for (int r = 0; r < 6; ++r) s[r * 32] = v[r];
+      float2 gx = s[6 * 32], gy = s[7 * 32];
+      if (l < 3) {  // one column for both feet; the CoM block takes it later
+        gy = both(gx.y);
+        gx = both(gx.x);
+      } else {
+        com_add2(cl, gx, gy);
       }
-    });
-    // CoM block: four partial sums, limbs first
+      add(v, gx, gy);
+    }
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+#pragma unroll
+      for (int k = 0; k <= i; ++k) {
+        L[tri(i, k)] = B[tri(i, k)].x;
+        L[tri(6 + i, 6 + k)] = B[tri(i, k)].y;
+      }
+      L[tri(18, i)] = C[i].x;
+      L[tri(18, 6 + i)] = C[i].y;
+      L[tri(19, i)] = C[6 + i].x;
+      L[tri(19, 6 + i)] = C[6 + i].y;
+    }
+    // right foot against left: the base's joints only
+    {
+      float X[36];
+#pragma unroll
+      for (int i = 0; i < 36; ++i) X[i] = i / 6 < 3 && i % 6 < 3 ? a.t.LR[i / 6 < 3 && i % 6 < 3 ? 3 * (i / 6) + i % 6 : 0] : 0.f;
+#pragma unroll 1
+      for (int b = 0; b < 3; ++b) {
+        float2 v[6];
+#pragma unroll
+        for (int r = 0; r < 6; ++r) v[r] = sm[(TP_BASE + 7 * b + r) * 32];
+#pragma unroll
+        for (int i = 0; i < 6; ++i)
+#pragma unroll
+          for (int k = 0; k < 6; ++k) X[6 * i + k] = fmaf(v[i].y, v[k].x, X[6 * i + k]);
+      }
+#pragma unroll
+      for (int i = 0; i < 36; ++i) L[tri(6 + i / 6, i % 6)] = X[i];
+    }
+    // CoM block: four partial sums (the arms, the left leg and the neck, the
+    // right leg), then the trunk joints, each in its partial
     float p[4][3];
 #pragma unroll
-    for (int g = 0; g < 4; ++g) p[g][0] = p[g][1] = p[g][2] = 0.f;
-    const auto add = [&](int g, float2 c) {
+    for (int i = 0; i < 3; ++i) {
+      p[0][i] = ca[i].x;
+      p[1][i] = ca[i].y;
+      p[2][i] = cl[i].x;
+      p[3][i] = cl[i].y;
+    }
+    const auto put = [&](int g, float2 c) {
       p[g][0] = fmaf(c.x, c.x, p[g][0]);
       p[g][1] = fmaf(c.y, c.x, p[g][1]);
       p[g][2] = fmaf(c.y, c.y, p[g][2]);
     };
-#pragma unroll
-    for (int i = 0; i < TR_ARM; ++i) {
-      add(0, at(TP_ARM + 4 * i + 3));
-      add(1, at(TP_ARM + 4 * (TR_ARM + i) + 3));
-    }
-#pragma unroll
-    for (int i = 0; i < TR_LEG; ++i) {
-      add(2, at(TP_LIMB + 4 * i + 3));
-      add(3, at(TP_LIMB + 4 * (TR_LEG + i) + 3));
-    }
-    add(2, at(TP_UP + 2));
-    add(2, at(TP_UP + 3));
+    put(2, at(TP_UP + 2));
+    put(2, at(TP_UP + 3));
     static_for<6>([&](auto JJ) {
       constexpr int j = decltype(JJ)::value;
-      if constexpr (j < 3) add(tree_part(j), jc[j]);
-      else add(tree_part(j), at(TP_BASE + 7 * (j - 3) + 6));
+      if constexpr (j < 3) put(tree_part(j), jc[j]);
+      else put(tree_part(j), at(TP_BASE + 7 * (j - 3) + 6));
     });
-    add(tree_part(TR_WAIST), at(TP_UP));
-    add(tree_part(TR_TORSO), at(TP_UP + 1));
+    put(tree_part(TR_WAIST), at(TP_UP));
+    put(tree_part(TR_TORSO), at(TP_UP + 1));
     L[tri(18, 18)] = __fadd_rn(__fadd_rn(p[0][0], p[1][0]), __fadd_rn(p[2][0], p[3][0]));
     L[tri(19, 18)] = __fadd_rn(__fadd_rn(p[0][1], p[1][1]), __fadd_rn(p[2][1], p[3][1]));
     L[tri(19, 19)] = __fadd_rn(__fadd_rn(p[0][2], p[1][2]), __fadd_rn(p[2][2], p[3][2]));
@@ -731,14 +845,17 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
   const bool go2 = act && !done;
   // y = A^{-1} F, then one refinement step with r = F - J (J^T y) - lambda y:
   // y += A^{-1} r; dq = J^T y in both passes (the second is the step)
-  float t[K], y[K], sp[4], db[3];
+  float t[K], yh[6], yc[2], db[3];
+  float2 yf[6];  // y of the feet (left, right); yh: of the hands; yc: of the CoM rows
+  float2 sa = make_float2(0.f, 0.f), sl = sa;  // |dq|^2: partial sums of the arms, of the legs
 #pragma unroll
-  for (int i = 0; i < K; ++i) {
-    t[i] = F[i];
-    y[i] = 0.f;
+  for (int i = 0; i < K; ++i) t[i] = F[i];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    yf[i] = make_float2(0.f, 0.f);
+    yh[i] = 0.f;
   }
-#pragma unroll
-  for (int g = 0; g < 4; ++g) sp[g] = 0.f;
+  yc[0] = yc[1] = 0.f;
 #pragma unroll
   for (int i = 0; i < 3; ++i) db[i] = 0.f;
 #pragma unroll 1
@@ -761,136 +878,109 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
       });
     });
 #pragma unroll
-    for (int i = 0; i < K; ++i) y[i] = __fadd_rn(y[i], t[i]);
+    for (int i = 0; i < 6; ++i) {
+      yf[i] = make_float2(__fadd_rn(yf[i].x, t[i]), __fadd_rn(yf[i].y, t[6 + i]));
+      yh[i] = __fadd_rn(yh[i], t[12 + i]);
+    }
+    yc[0] = __fadd_rn(yc[0], t[18]);
+    yc[1] = __fadd_rn(yc[1], t[19]);
     // per joint: dq_j = J_j . y and, for the refinement, r += J_j dq_j
-    float r[18], pc[4][2], dqb[6];
-#pragma unroll
-    for (int i = 0; i < 18; ++i) r[i] = 0.f;
-#pragma unroll
-    for (int g = 0; g < 4; ++g) pc[g][0] = pc[g][1] = sp[g] = 0.f;
     const bool last = pass == 1;
-    const auto step = [&](int g, float d, float2 c) -> float {  // CoM partial sums, the scaled step
+    float2 rf[6], pl[2];  // feet: r; CoM partial sums of the legs, of the arms
+    float pa[2][2];
+    float dqb[6], rh[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      rf[i] = make_float2(0.f, 0.f);
+      rh[i] = 0.f;
+    }
+    sa = sl = pl[0] = pl[1] = make_float2(0.f, 0.f);
+    pa[0][0] = pa[0][1] = pa[1][0] = pa[1][1] = 0.f;
+    const auto com_dot = [&](float2 c, float acc) { return fmaf(c.x, yc[0], fmaf(c.y, yc[1], acc)); };
+    // base: prismatic columns are constants (their rotational rows zero)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      float acc = 0.f;
+      acc = fmaf(a.t.jt[i][0].x, yf[0].x, fmaf(a.t.jt[i][1].x, yf[1].x, acc));
+      acc = fmaf(a.t.jt[i][2].x, yf[2].x, acc);
+      acc = fmaf(a.t.jt[i][0].y, yf[0].y, fmaf(a.t.jt[i][1].y, yf[1].y, acc));
+      acc = fmaf(a.t.jt[i][2].y, yf[2].y, acc);
+      dqb[i] = com_dot(jc[i], acc);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) rf[k] = __ffma2_rn(a.t.jt[i][k], both(dqb[i]), rf[k]);
+    }
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      float2 v[6];
+#pragma unroll
+      for (int r = 0; r < 6; ++r) v[r] = at(TP_BASE + 7 * b + r);
+      float acc = 0.f;
+#pragma unroll
+      for (int r = 0; r < 6; r += 2) acc = fmaf(v[r].x, yf[r].x, fmaf(v[r + 1].x, yf[r + 1].x, acc));
+#pragma unroll
+      for (int r = 0; r < 6; r += 2) acc = fmaf(v[r].y, yf[r].y, fmaf(v[r + 1].y, yf[r + 1].y, acc));
+      dqb[3 + b] = com_dot(at(TP_BASE + 7 * b + 6), acc);
+#pragma unroll
+      for (int r = 0; r < 6; ++r) rf[r] = __ffma2_rn(v[r], both(dqb[3 + b]), rf[r]);
+    }
+    // limbs: the scaled step of the last pass stays in the joint's first slot
+    {
+      float2 *leg = sm + TP_LEG * 32;
+#pragma unroll 1
+      for (int l = 0; l < TR_LEG; ++l, leg += 8 * 32) {
+        float2 v[6];
+#pragma unroll
+        for (int r = 0; r < 6; ++r) v[r] = leg[r * 32];
+        const float2 gx = leg[6 * 32], gy = leg[7 * 32];
+        float2 d = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int r = 0; r < 6; r += 2) d = __ffma2_rn(v[r], yf[r], __ffma2_rn(v[r + 1], yf[r + 1], d));
+        d = __ffma2_rn(gx, both(yc[0]), __ffma2_rn(gy, both(yc[1]), d));
+        pl[0] = __ffma2_rn(gx, d, pl[0]);
+        pl[1] = __ffma2_rn(gy, d, pl[1]);
+#pragma unroll
+        for (int r = 0; r < 6; ++r) rf[r] = __ffma2_rn(v[r], d, rf[r]);
+        const float2 e = __fmul2_rn(d, both(a.alpha));
+        sl = __ffma2_rn(e, e, sl);
+        if (last) leg[0] = e;
+      }
+    }
+    // the arms one after the other (r sums the left arm's terms first)
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      float sq = 0.f;
+      float *arm = reinterpret_cast<float *>(sm + TP_ARM * 32) + s;
+#pragma unroll 1
+      for (int l = 0; l < TR_ARM; ++l, arm += 8 * 64) {
+        float v[6];
+#pragma unroll
+        for (int r = 0; r < 6; ++r) v[r] = arm[r * 64];
+        const float gx = arm[6 * 64], gy = arm[7 * 64];
+        float d = 0.f;
+#pragma unroll
+        for (int r = 0; r < 6; r += 2) d = fmaf(v[r], yh[r], fmaf(v[r + 1], yh[r + 1], d));
+        d = fmaf(gx, yc[0], fmaf(gy, yc[1], d));
+        pa[s][0] = fmaf(gx, d, pa[s][0]);
+        pa[s][1] = fmaf(gy, d, pa[s][1]);
+#pragma unroll
+        for (int r = 0; r < 6; ++r) rh[r] = fmaf(v[r], d, rh[r]);
+        const float e = __fmul_rn(d, a.alpha);
+        sq = fmaf(e, e, sq);
+        if (last) arm[0] = e;
+      }
+      if (s == 0) sa.x = sq;
+      else sa.y = sq;
+    }
+    // neck, then the trunk joints, each in its partial sum
+    float pc[4][2] = {{pa[0][0], pa[0][1]}, {pa[1][0], pa[1][1]}, {pl[0].x, pl[1].x}, {pl[0].y, pl[1].y}};
+    float sp[4] = {sa.x, sa.y, sl.x, sl.y};
+    const auto step = [&](int g, float d, float2 c) -> float {
       pc[g][0] = fmaf(c.x, d, pc[g][0]);
       pc[g][1] = fmaf(c.y, d, pc[g][1]);
       const float e = __fmul_rn(d, a.alpha);
       sp[g] = fmaf(e, e, sp[g]);
       return e;
     };
-    const auto com_dot = [&](float2 c, float acc) { return fmaf(c.x, y[18], fmaf(c.y, y[19], acc)); };
-    const auto seg_dot = [&](const float2 (&v)[3], const float (&w)[6], float acc) {
-#pragma unroll
-      for (int i = 0; i < 3; ++i) acc = fmaf(v[i].x, w[2 * i], fmaf(v[i].y, w[2 * i + 1], acc));
-      return acc;
-    };
-    const auto seg_add = [&](const float2 (&v)[3], float d, float (&w)[6]) {
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        w[2 * i] = fmaf(v[i].x, d, w[2 * i]);
-        w[2 * i + 1] = fmaf(v[i].y, d, w[2 * i + 1]);
-      }
-    };
-    float yf[2][6], rf[2][6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      yf[0][i] = y[i];
-      yf[1][i] = y[6 + i];
-      rf[0][i] = rf[1][i] = 0.f;
-    }
-    // base: prismatic columns are constants (their rotational rows zero)
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      float acc = 0.f;
-#pragma unroll
-      for (int s = 0; s < 2; ++s) {
-        acc = fmaf(a.t.jt[s][i][0], yf[s][0], fmaf(a.t.jt[s][i][1], yf[s][1], acc));
-        acc = fmaf(a.t.jt[s][i][2], yf[s][2], acc);
-      }
-      acc = com_dot(jc[i], acc);
-      dqb[i] = acc;
-#pragma unroll
-      for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) rf[s][k] = fmaf(a.t.jt[s][i][k], acc, rf[s][k]);
-    }
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      const int e = TP_BASE + 7 * b;
-      const float2 vl[3] = {at(e), at(e + 1), at(e + 2)}, vr[3] = {at(e + 3), at(e + 4), at(e + 5)};
-      const float d = com_dot(at(e + 6), seg_dot(vr, yf[1], seg_dot(vl, yf[0], 0.f)));
-      dqb[3 + b] = d;
-      seg_add(vl, d, rf[0]);
-      seg_add(vr, d, rf[1]);
-    }
-#pragma unroll 1
-    for (int s = 0; s < 2; ++s) {  // legs
-      float w[6], ra[6];
-#pragma unroll
-      for (int i = 0; i < 6; ++i) {
-        w[i] = s == 0 ? yf[0][i] : yf[1][i];
-        ra[i] = s == 0 ? rf[0][i] : rf[1][i];
-      }
-      pc[2][0] = pc[2][1] = sp[2] = 0.f;
-      float2 *leg = sm + (TP_LIMB + 4 * TR_LEG * s) * 32;
-#pragma unroll
-      for (int i = 0; i < TR_LEG; ++i) {
-        const float2 v[3] = {leg[4 * i * 32], leg[(4 * i + 1) * 32], leg[(4 * i + 2) * 32]};
-        const float2 c = leg[(4 * i + 3) * 32];
-        const float d = com_dot(c, seg_dot(v, w, 0.f));
-        seg_add(v, d, ra);
-        const float e = step(2, d, c);
-        if (last) leg[4 * i * 32].x = e;
-      }
-      if (s == 0) {  // the left leg's sums move on; partial 2 starts over for the right leg
-#pragma unroll
-        for (int i = 0; i < 6; ++i) r[i] = ra[i];
-        pc[3][0] = pc[2][0];
-        pc[3][1] = pc[2][1];
-        sp[3] = sp[2];
-      } else {
-#pragma unroll
-        for (int i = 0; i < 6; ++i) r[6 + i] = ra[i];
-      }
-    }
-    // partial 2 is the left leg's, 3 the right leg's
-    {
-      const float u0 = pc[2][0], u1 = pc[2][1], u2 = sp[2];
-      pc[2][0] = pc[3][0];
-      pc[2][1] = pc[3][1];
-      sp[2] = sp[3];
-      pc[3][0] = u0;
-      pc[3][1] = u1;
-      sp[3] = u2;
-    }
-    {
-      float w[6], ra[6];
-#pragma unroll
-      for (int i = 0; i < 6; ++i) {
-        w[i] = y[12 + i];
-        ra[i] = 0.f;
-      }
-#pragma unroll 1
-      for (int s = 0; s < 2; ++s) {  // arms
-        pc[1][0] = pc[1][1] = sp[1] = 0.f;
-        float2 *arm = sm + (TP_ARM + 4 * TR_ARM * s) * 32;
-#pragma unroll
-        for (int i = 0; i < TR_ARM; ++i) {
-          const float2 v[3] = {arm[4 * i * 32], arm[(4 * i + 1) * 32], arm[(4 * i + 2) * 32]};
-          const float2 c = arm[(4 * i + 3) * 32];
-          const float d = com_dot(c, seg_dot(v, w, 0.f));
-          seg_add(v, d, ra);
-          const float e = step(1, d, c);
-          if (last) arm[4 * i * 32].x = e;
-        }
-        if (s == 0) {
-          pc[0][0] = pc[1][0];
-          pc[0][1] = pc[1][1];
-          sp[0] = sp[1];
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < 6; ++i) r[12 + i] = ra[i];
-    }
-    // neck, then the trunk joints, each in its partial sum
     static_for<4>([&](auto II) {
       constexpr int i = (decltype(II)::value + 2) % 4;  // neck (2, 3), then waist (0) and torso (1)
       if constexpr (i == 0) {
@@ -908,17 +998,23 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
       const float e = step(tree_part(TR_WAIST + i), com_dot(c, 0.f), c);
       if (last) at(TP_UP + i).x = e;
     });
+    sa = make_float2(sp[0], sp[1]);
+    sl = make_float2(sp[2], sp[3]);
     if (last) break;
 #pragma unroll
-    for (int i = 0; i < 18; ++i) t[i] = fmaf(-a.lambda, y[i], __fadd_rn(F[i], -r[i]));
+    for (int i = 0; i < 6; ++i) {
+      t[i] = fmaf(-a.lambda, yf[i].x, __fadd_rn(F[i], -rf[i].x));
+      t[6 + i] = fmaf(-a.lambda, yf[i].y, __fadd_rn(F[6 + i], -rf[i].y));
+      t[12 + i] = fmaf(-a.lambda, yh[i], __fadd_rn(F[12 + i], -rh[i]));
+    }
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const float s = __fadd_rn(__fadd_rn(pc[0][i], pc[1][i]), __fadd_rn(pc[2][i], pc[3][i]));
-      t[18 + i] = fmaf(-a.lambda, y[18 + i], __fadd_rn(F[18 + i], -s));
+      t[18 + i] = fmaf(-a.lambda, yc[i], __fadd_rn(F[18 + i], -s));
     }
   }
   // MaxDistance, update (the scaled steps lie in the first word of each joint's slot)
-  const float s2 = __fadd_rn(__fadd_rn(sp[0], sp[1]), __fadd_rn(sp[2], sp[3]));
+  const float s2 = __fadd_rn(__fadd_rn(sa.x, sa.y), __fadd_rn(sl.x, sl.y));
   if (go2 && a.max_step2 > 0.f && s2 > a.max_step2) {
     fl |= FL_DIV;
     done = true;
@@ -932,9 +1028,17 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
 #pragma unroll
     for (int i = 0; i < 4; ++i) q[TR_WAIST + i] = __fadd_rn(q[TR_WAIST + i], -at(TP_UP + i).x);
 #pragma unroll
-    for (int l = 0; l < 2 * TR_LEG; ++l) q[TR_LEG0 + l] = __fadd_rn(q[TR_LEG0 + l], -at(TP_LIMB + 4 * l).x);
+    for (int l = 0; l < TR_LEG; ++l) {
+      const float2 e = at(TP_LEG + 8 * l);
+      q[TR_LEG0 + l] = __fadd_rn(q[TR_LEG0 + l], -e.x);
+      q[TR_LEG0 + TR_LEG + l] = __fadd_rn(q[TR_LEG0 + TR_LEG + l], -e.y);
+    }
 #pragma unroll
-    for (int l = 0; l < 2 * TR_ARM; ++l) q[TR_ARM0 + l] = __fadd_rn(q[TR_ARM0 + l], -at(TP_ARM + 4 * l).x);
+    for (int l = 0; l < TR_ARM; ++l) {
+      const float2 e = at(TP_ARM + 8 * l);
+      q[TR_ARM0 + l] = __fadd_rn(q[TR_ARM0 + l], -e.x);
+      q[TR_ARM0 + TR_ARM + l] = __fadd_rn(q[TR_ARM0 + TR_ARM + l], -e.y);
+    }
     ++it;
     fl &= ~FL_INT_FORCE;
     if (!(s2 <= FLT_MAX)) {
@@ -951,7 +1055,7 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
 // FP64 acceptances; those sent back for another FP32 step wait likewise (one
 // per lane).  A 32-word scratch per warp routes them.  An acceptance always
 // runs once a warp could not hold another iteration's 32 configurations, or
-// has nothing else to do, with or without the token.
+// the team has nothing else to do, with or without the token.
 constexpr int TREE_WARPS = 7;
 constexpr int TREE_TEAM = 4;
 constexpr int TREE_ACCEPT_MIN = 20;
@@ -974,6 +1078,8 @@ __global__ void __launch_bounds__(TREE_WARPS * 32, 1) k_project_tree(const __gri
   const int warps = blockDim.x >> 5, team0 = wib < TREE_TEAM ? 0 : TREE_TEAM;  // first warp of the team
   const TreeTeam team{1 + (team0 > 0), 32 * (team0 > 0 ? warps - TREE_TEAM : min(warps, TREE_TEAM))};
   long long qn = 0, qe = 0;  // warp-local queue [qn, qe)
+  long long an = 0, ae = 0;  // the chunk after it, claimed ahead and on its way into L2
+  const long long margin = 2ll * a.chunk * gridDim.x * warps;
   bool more = true;
   bool act = false;
   int item = 0;
@@ -988,21 +1094,41 @@ __global__ void __launch_bounds__(TREE_WARPS * 32, 1) k_project_tree(const __gri
   while (true) {
     // refill idle lanes: retries first, then new work
     const unsigned idle = __ballot_sync(FULL, !act);
-    if (idle != 0u && (nret > 0 || qn < qe || more)) {
+    if (idle != 0u && (nret > 0 || qn < qe || an < ae || more)) {
       const int n_idle = __popc(idle);
       const int from_r = n_idle < nret ? n_idle : nret;
       const int need = n_idle - from_r;
       const long long avail = qe - qn;
       long long b0 = 0, b1 = 0;
-      if (need > 0 && avail < need && more) {
+      const auto claim = [&](long long &lo, long long &hi) {
         unsigned long long b = 0;
         if (lane == 0) b = atomicAdd(a.counter, static_cast<unsigned long long>(a.chunk));
         b = __shfl_sync(FULL, b, 0);
         if (static_cast<long long>(b) >= a.total) {
           more = false;
         } else {
-          b0 = static_cast<long long>(b);
-          b1 = b0 + a.chunk < a.total ? b0 + a.chunk : a.total;
+          lo = static_cast<long long>(b);
+          hi = lo + a.chunk < a.total ? lo + a.chunk : a.total;
+        }
+      };
+      if (need > 0 && avail < need) {
+        if (an < ae) {
+          b0 = an;
+          b1 = ae;
+          an = ae = 0;
+        } else if (more) {
+          claim(b0, b1);
+        }
+        // while much work is left, the next chunk's rows start towards L2 now
+        // (not near the end, where a chunk held back would leave others idle)
+        if (more && b1 + margin < a.total) {
+          claim(an, ae);
+          if (an < ae)
+            for (int j = lane; j < D; j += 32) {
+              const float *row = a.src.q + j * a.src.ld;
+              asm volatile("prefetch.global.L2 [%0];" ::"l"(row + an));
+              asm volatile("prefetch.global.L2 [%0];" ::"l"(row + ae - 1));
+            }
         }
       }
       const int rank_all = __popc(idle & ((1u << lane) - 1u));
@@ -1078,13 +1204,14 @@ __global__ void __launch_bounds__(TREE_WARPS * 32, 1) k_project_tree(const __gri
       if (done) act = false;
       pend += nf;
     }
-    const bool drained = !__any_sync(FULL, act) && qn >= qe && !more && nret == 0;
+    const bool drained = !__any_sync(FULL, act) && qn >= qe && an >= ae && !more && nret == 0;
     // FP64 acceptance, one configuration per lane, 32 at a time; a failed
     // acceptance with steps left goes back to the FP32 loop
     bool accept = false, token = false;
-    if (team.any(pend >= 32 || (drained && pend > 0))) {
+    const bool full = team.any(pend > 32 * (TREE_SLOTS - 1)), wait = team.any(pend < 32 && !drained);
+    if (full || !wait) {
       if (wib == team0 && lane == 0) token = atomicCAS(&fp64_taken, 0, 1) == 0;
-      accept = team.any(token || pend > 32 * (TREE_SLOTS - 1) || drained);
+      accept = full || team.any(token || drained);
     }
     if (accept && pend > 0 && (pend >= TREE_ACCEPT_MIN || drained)) {
       const int take = pend < 32 ? pend : 32;

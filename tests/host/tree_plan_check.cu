@@ -27,8 +27,8 @@ template <class P> int check() {
   }
   int used[TREE_PAIRS] = {0};
   auto mark = [&](int e, int n) { for (int i = 0; i < n; ++i) { if (e + i < 0 || e + i >= TREE_PAIRS) bad++; else used[e + i]++; } };
-  for (int l = 0; l < 2 * TR_LEG; ++l) mark(TP_LIMB + 4 * l, 4);
-  for (int l = 0; l < 2 * TR_ARM; ++l) mark(TP_ARM + 4 * l, 4);
+  for (int l = 0; l < TR_LEG; ++l) mark(TP_LEG + 8 * l, 8);
+  for (int l = 0; l < TR_ARM; ++l) mark(TP_ARM + 8 * l, 8);
   for (int b = 0; b < 3; ++b) mark(TP_BASE + 7 * b, 7);
   mark(TP_UP, 4);
   for (int e = 0; e < TREE_PAIRS; ++e) if (used[e] != 1) bad++, printf("pair %d used %d times\n", e, used[e]);
@@ -62,15 +62,15 @@ template <class P> int check() {
   for (int s = 0; s < 2; ++s) for (int r = 0; r < 3; ++r) for (int c = 0; c < 3; ++c) {
     double ll = 0, lr = 0, cl = 0;
     for (int i = 0; i < 3; ++i) {
-      err = std::max(err, std::fabs(t.jt[s][i][r] - jt[s][i][r]));
+      err = std::max(err, std::fabs((s ? t.jt[i][r].y : t.jt[i][r].x) - jt[s][i][r]));
       if (r < 2) err = std::max(err, std::fabs(t.jc[i][r] - jc[i][r]));
       ll += jt[s][i][r] * jt[s][i][c];
       lr += jt[1][i][r] * jt[0][i][c];
       if (r < 2) cl += jc[i][r] * jt[s][i][c];
     }
-    if (c <= r) err = std::max(err, std::fabs(t.LL[s][tri(r, c)] - ll));
+    if (c <= r) err = std::max(err, std::fabs((s ? t.LL[tri(r, c)].y : t.LL[tri(r, c)].x) - ll));
     err = std::max(err, std::fabs(t.LR[3 * r + c] - lr));
-    if (r < 2) err = std::max(err, std::fabs(t.CL[s][3 * r + c] - cl));
+    if (r < 2) err = std::max(err, std::fabs((s ? t.CL[3 * r + c].y : t.CL[3 * r + c].x) - cl));
   }
   if (!(err < 2e-6)) bad++, printf("constants off by %g\n", err);  // a few roundings of O(1) values in FP32
   printf("%s: %d problems\n", P::name, bad);

@@ -12,7 +12,8 @@ def test_tree_kernel_structure_matches_the_plan():
     with tempfile.TemporaryDirectory() as d:
         exe = os.path.join(d, "tree_plan_check")
         src = os.path.join(ROOT, "tests", "host", "tree_plan_check.cu")
-        r = subprocess.run([_nvcc(), "-std=c++17", "--expt-relaxed-constexpr", "-O1", "-I",
+        r = subprocess.run([_nvcc(), "-gencode", "arch=compute_103a,code=sm_103a", "-std=c++17",
+                            "--expt-relaxed-constexpr", "-O1", "-I",
                             os.path.join(ROOT, "include"), src, "-o", exe], capture_output=True, text=True)
         assert r.returncode == 0, r.stderr[-3000:]
         r = subprocess.run([exe], capture_output=True, text=True, timeout=120)
