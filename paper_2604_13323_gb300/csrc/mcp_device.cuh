@@ -77,6 +77,12 @@ enum : uint32_t {
   FL_CONV = 1, FL_CAP = 2, FL_DIV = 4, FL_NONFINITE = 8, FL_RESOLVE = 16, FL_ACCEPT_FAIL = 32, FL_LIMITS = 64
 };
 
+constexpr unsigned FULL = 0xffffffffu;
+// internal flag bits (never written out)
+constexpr uint32_t FL_INT_FP32CONV = 1u << 8;   // FP32 residual passed; FP64 check pending
+constexpr uint32_t FL_INT_NEEDS_F64 = 1u << 9;  // FP32 pivot below threshold: continue in FP64
+constexpr uint32_t FL_INT_FORCE = 1u << 10;     // FP64 acceptance failed: one FP32 step before the next test
+
 // Model data in one precision.  3x4 transforms are row-major (column 3 = translation).
 template <typename T>
 struct ModelT {

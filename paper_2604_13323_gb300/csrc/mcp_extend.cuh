@@ -94,15 +94,19 @@ __device__ __noinline__ bool accept_regs(const A &a, float (&q)[P::D], int &it, 
 // Projects the point of every active lane (warp-convergent: all lanes call
 // it).  Out of line: the extension calls it at three places and one copy keeps
 // the kernel within the instruction cache.
+// slots: this lane's shared memory of the step (classes that keep their Jacobian there).
 template <class P, class A>
-__device__ __noinline__ void project_lanes(const A &a, float (&q)[P::D], bool active, int &it, uint32_t &fl) {
+__device__ __noinline__ void project_lanes(const A &a, float2 *slots, float (&q)[P::D], bool active, int &it, uint32_t &fl) {
   it = 0;
   fl = 0;
   bool done = !active;
   bool final_ = !active;  // accepted (or inactive)
   while (true) {
     while (__any_sync(FULL, !done)) {
-      if (!done) done = newton_iter_f32<P>(a, q, it, fl);
+      if (!done) {
+        if constexpr (iter_smem<P, FORM_STACKED>() > 0) done = dual_iter_f32<P>(a, slots, q, it, fl);
+        else done = newton_iter_f32<P>(a, q, it, fl);
+      }
     }
     bool again = false;
     if (!final_) {
@@ -151,7 +155,9 @@ __global__ void __launch_bounds__(W * 32) k_extend(const __grid_constant__ ExtAr
   constexpr int NG = 32 / G;
   static_assert(G == 8 || G == 16 || G == 32, "groups of 8, 16 or 32 lanes");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float4 *s_pair = reinterpret_cast<float4 *>(smem_raw);
+  constexpr int SLOT_BYTES = iter_smem<P, FORM_STACKED>();  // per thread, a multiple of 16 bytes per warp
+  float2 *slots = reinterpret_cast<float2 *>(smem_raw) + (threadIdx.x >> 5) * (SLOT_BYTES / 8 * 32) + (threadIdx.x & 31);
+  float4 *s_pair = reinterpret_cast<float4 *>(smem_raw + W * 32 * SLOT_BYTES);
   const float *s_box = stage_obstacles(a.obs, a.n_obs, a.box, a.n_box, s_pair);
   __syncthreads();
   const int lane = threadIdx.x & 31;
@@ -217,7 +223,7 @@ __global__ void __launch_bounds__(W * 32) k_extend(const __grid_constant__ ExtAr
         p[j] = fmaf(ep, v[j], fmaf(dist, v[j], qs[j]));
       }
     }
-    project_lanes<P>(a, p, alive && act, it, fl);
+    project_lanes<P>(a, slots, p, alive && act, it, fl);
     if (alive && act) work += it;
     {
       constexpr unsigned BIG = 0xffffffffu;
@@ -261,7 +267,7 @@ __global__ void __launch_bounds__(W * 32) k_extend(const __grid_constant__ ExtAr
 #pragma unroll
       for (int j = 0; j < D; ++j) xq[j] = fmaf(tk, qp[j] - qs[j], qs[j]);
     }
-    project_lanes<P>(a, xq, alive && act, it, fl);
+    project_lanes<P>(a, slots, xq, alive && act, it, fl);
     if (alive && act) work += it;
     const bool unconv = gballot(act && !(fl & FL_CONV)) != 0u;  // every lane votes
     if (alive && unconv) {
@@ -338,7 +344,7 @@ __global__ void __launch_bounds__(W * 32) k_extend(const __grid_constant__ ExtAr
           if (in) next[pos * D + j] = lo;
           mq[j] = 0.5f * (lo + hi);
         }
-        project_lanes<P>(a, mq, w, it, fl);
+        project_lanes<P>(a, slots, mq, w, it, fl);
         if (w) work += it;
         int code = 0;
         if (w) {
@@ -392,7 +398,7 @@ template <class P, int G>
 cudaError_t launch_extend_g(const HostModel &hm, const ExtCall &c, ExtArgs<P> &a, int *launches) {
   constexpr int W = 2;
   auto kern = k_extend<P, W, G>;
-  const size_t smem = obs_smem_bytes(hm.n_obs, hm.n_box);
+  const size_t smem = obs_smem_bytes(hm.n_obs, hm.n_box) + static_cast<size_t>(W) * 32 * iter_smem<P, FORM_STACKED>();
   cudaError_t err = cudaSuccess;
   if (smem > 48 * 1024) err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (err != cudaSuccess) return err;

@@ -14,16 +14,11 @@
 
 #include "mcp_accept.cuh"
 #include "mcp_device.cuh"
+#include "mcp_dual.cuh"
 #include "mcp_internal.h"
 #include "mcp_problems.cuh"
 
 namespace mcp {
-
-constexpr unsigned FULL = 0xffffffffu;
-// internal flag bits (never written out)
-constexpr uint32_t FL_INT_FP32CONV = 1u << 8;   // FP32 residual passed; FP64 check pending
-constexpr uint32_t FL_INT_NEEDS_F64 = 1u << 9;  // FP32 pivot below threshold: continue in FP64
-constexpr uint32_t FL_INT_FORCE = 1u << 10;     // FP64 acceptance failed: one FP32 step before the next test
 
 // Forms of getDescentStep (Alg. 2): the stacked inner step J^T (J J^T + lambda I)^-1 F,
 // one inner step per constraint in turn (cyclic), or the stacked outer step
@@ -1277,21 +1272,29 @@ __global__ void __launch_bounds__(128) k_check_f64(const __grid_constant__ Check
 // ---------------------------------------------------------------------------
 // Register budget of the persistent kernel: what the FP32 loop needs (the FP64
 // finishing path may spill; it is rare).  Sets the resident blocks per SM.
-template <class P>
+template <class P, int FORM>
 __host__ __device__ constexpr int reg_cap() {
-  return (P::D <= 7 && kdim<P>() <= 2) ? 128 : 168;
+  return ((P::D <= 7 && kdim<P>() <= 2) || (FORM == FORM_STACKED && dual_layout_matches<P>())) ? 128 : 168;
 }
-template <class P, int TPB>
+template <class P, int TPB, int FORM>
 __host__ __device__ constexpr int min_blocks() {
-  return 65536 / (TPB * reg_cap<P>()) > 0 ? 65536 / (TPB * reg_cap<P>()) : 1;
+  return 65536 / (TPB * reg_cap<P, FORM>()) > 0 ? 65536 / (TPB * reg_cap<P, FORM>()) : 1;
 }
 
 // Configurations a warp can hold for an FP32 retry after a failed FP64
 // acceptance (beyond this the acceptance finishes them in FP64 itself).
 constexpr int RETRY_CAP = 32;
 
+// Bytes of the Newton step's slots in shared memory (classes whose stacked
+// step keeps its Jacobian there), per thread.
+template <class P, int FORM>
+__host__ __device__ constexpr int iter_smem() {
+  if constexpr (FORM == FORM_STACKED) return dual_layout_matches<P>() ? DUAL_PAIRS * static_cast<int>(sizeof(float2)) : 0;
+  else return 0;
+}
+
 template <class P, class Src, int TPB, int FORM, bool CHK>
-__global__ void __launch_bounds__(TPB, (min_blocks<P, TPB>())) k_project_f32(const __grid_constant__ ProjArgs<P, Src> a) {
+__global__ void __launch_bounds__(TPB, (min_blocks<P, TPB, FORM>())) k_project_f32(const __grid_constant__ ProjArgs<P, Src> a) {
   constexpr int D = P::D;
   constexpr int W = TPB / 32;
   __shared__ long long s_item[W][64];
@@ -1299,7 +1302,10 @@ __global__ void __launch_bounds__(TPB, (min_blocks<P, TPB>())) k_project_f32(con
   __shared__ long long s_ritem[W][RETRY_CAP];  // sent back to the FP32 loop by the acceptance
   __shared__ uint32_t s_rmeta[W][RETRY_CAP];
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float4 *s_pair = reinterpret_cast<float4 *>(smem_raw);
+  // the step's slots first (a multiple of 16 bytes), then the obstacles
+  [[maybe_unused]] float2 *slots = reinterpret_cast<float2 *>(smem_raw) +
+                                   (threadIdx.x >> 5) * (iter_smem<P, FORM>() / 8 * 32) + (threadIdx.x & 31);
+  float4 *s_pair = reinterpret_cast<float4 *>(smem_raw + TPB * iter_smem<P, FORM>());
   const float *s_box = nullptr;
   if constexpr (CHK) {  // obstacles of the fused check, staged once per block
     s_box = stage_obstacles(a.obs, a.n_obs, a.box, a.n_box, s_pair);
@@ -1379,6 +1385,7 @@ __global__ void __launch_bounds__(TPB, (min_blocks<P, TPB>())) k_project_f32(con
     bool done = false;
     if (act) {
       if constexpr (FORM == FORM_CYCLIC) done = cyclic_iter_f32<P>(a, q, it, fl);
+      else if constexpr (iter_smem<P, FORM>() > 0) done = dual_iter_f32<P>(a, slots, q, it, fl);
       else done = newton_iter_f32<P, ProjArgs<P, Src>, FORM == FORM_OUTER>(a, q, it, fl);
     }
     // (3) park finished lanes
@@ -1774,13 +1781,18 @@ cudaError_t launch_persistent(const HostModel &hm, const ProjCall &c, const Src 
   a.n_box = CHK ? hm.n_box : 0;
   a.hit = c.hit;
   a.pairs = c.pairs;
-  const size_t smem = CHK ? obs_smem_bytes(hm.n_obs, hm.n_box) : 0;
+  const size_t smem = (CHK ? obs_smem_bytes(hm.n_obs, hm.n_box) : 0) + static_cast<size_t>(TPB) * iter_smem<P, FORM>();
+  auto kern = k_project_f32<P, Src, TPB, FORM, CHK>;
+  if (smem > 40 * 1024) {  // with the kernel's static arrays above the 48 KB a launch gets unasked
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+  }
   const long long warps_needed = (c.total + 31) / 32;
   long long blocks = static_cast<long long>(hm.sm_count) * c.tune.blocks_per_sm;
   const long long max_useful = (warps_needed + (TPB / 32) - 1) / (TPB / 32);
   if (blocks > max_useful) blocks = max_useful;
   if (blocks < 1) blocks = 1;
-  k_project_f32<P, Src, TPB, FORM, CHK><<<static_cast<unsigned>(blocks), TPB, smem, c.stream>>>(a);
+  kern<<<static_cast<unsigned>(blocks), TPB, smem, c.stream>>>(a);
   return cudaGetLastError();
 }
 
