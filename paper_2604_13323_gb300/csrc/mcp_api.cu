@@ -284,8 +284,9 @@ __global__ void k_resolve(const __grid_constant__ ResolveIn in, ResolveOut *out)
 
 // Obstacle preparation (one block): centroid of the obstacle centres (FP64),
 // then per obstacle sphere the FP32 records of the expanded overlap test in
-// the shifted frame: (-2c, |c|^2 - r^2), (-2r, 0, 0, 0); after them, one
-// record of the same form per chunk of OBS_CHUNK consecutive obstacles: a
+// the shifted frame (-2c, |c|^2 - r^2, -2r), already in the pairs that the
+// kernels hold in shared memory (obs_rec); after them, one record of the same
+// form per chunk of OBS_CHUNK consecutive obstacles: a
 // sphere around the chunk (centre the mean of its centres, radius the largest
 // |c_o - c| + r_o plus 1e-4 m, which keeps the FP32 test of the chunk
 // conservative); boxes shifted.
@@ -321,16 +322,19 @@ __global__ void k_prep_obstacles(const double *obs, int n_obs, const double *box
     origin[1] = oy;
     origin[2] = oz;
   }
+  // record o in the layout of shared memory: two records per 12 floats
+  const auto put = [&](int o, double gx, double gy, double gz, double gw, double g2) {
+    float *f = obs32 + 12 * (o >> 1) + (o & 1);
+    f[0] = static_cast<float>(gx);
+    f[2] = static_cast<float>(gy);
+    f[4] = static_cast<float>(gz);
+    f[6] = static_cast<float>(gw);
+    f[8] = static_cast<float>(g2);
+    f[10] = 0.f;
+  };
   for (int o = t; o < n_obs; o += blockDim.x) {
     const double cx = obs[4 * o] - ox, cy = obs[4 * o + 1] - oy, cz = obs[4 * o + 2] - oz, r = obs[4 * o + 3];
-    obs32[8 * o + 0] = static_cast<float>(-2.0 * cx);
-    obs32[8 * o + 1] = static_cast<float>(-2.0 * cy);
-    obs32[8 * o + 2] = static_cast<float>(-2.0 * cz);
-    obs32[8 * o + 3] = static_cast<float>(cx * cx + cy * cy + cz * cz - r * r);
-    obs32[8 * o + 4] = static_cast<float>(-2.0 * r);
-    obs32[8 * o + 5] = 0.f;
-    obs32[8 * o + 6] = 0.f;
-    obs32[8 * o + 7] = 0.f;
+    put(o, -2.0 * cx, -2.0 * cy, -2.0 * cz, cx * cx + cy * cy + cz * cz - r * r, -2.0 * r);
   }
   for (int k = t; k < obs_chunks(n_obs); k += blockDim.x) {
     const int o0 = k * OBS_CHUNK, o1 = o0 + OBS_CHUNK < n_obs ? o0 + OBS_CHUNK : n_obs;
@@ -350,14 +354,11 @@ __global__ void k_prep_obstacles(const double *obs, int n_obs, const double *box
       rad = e > rad ? e : rad;
     }
     rad += 1e-4;
-    float *rec = obs32 + 8 * (n_obs + k);
-    rec[0] = static_cast<float>(-2.0 * mx);
-    rec[1] = static_cast<float>(-2.0 * my);
-    rec[2] = static_cast<float>(-2.0 * mz);
-    rec[3] = static_cast<float>(mx * mx + my * my + mz * mz - rad * rad);
-    rec[4] = static_cast<float>(-2.0 * rad);
-    rec[5] = rec[6] = rec[7] = 0.f;
+    put(2 * obs_pairs(n_obs) + k, -2.0 * mx, -2.0 * my, -2.0 * mz, mx * mx + my * my + mz * mz - rad * rad, -2.0 * rad);
   }
+  // the second half of an odd count's last pair never overlaps
+  if (t == 0 && n_obs % 2) put(n_obs, 0.0, 0.0, 0.0, 1e30, 0.0);
+  if (t == 0 && obs_chunks(n_obs) % 2) put(2 * obs_pairs(n_obs) + obs_chunks(n_obs), 0.0, 0.0, 0.0, 1e30, 0.0);
   for (int b = t; b < n_box; b += blockDim.x) {
     box32[6 * b + 0] = static_cast<float>(box[6 * b + 0] - ox);
     box32[6 * b + 1] = static_cast<float>(box[6 * b + 1] - oy);
@@ -1076,8 +1077,8 @@ mcp_status mcp_load_obstacles(mcp_ctx *ctx, const double *spheres, int32_t n_sph
     for (int o = 0; o < n_spheres; ++o)
       for (int e = 0; e < 4; ++e) sorted[4 * static_cast<size_t>(o) + e] = spheres[4 * key[static_cast<size_t>(o)].second + e];
   }
-  const size_t n_rec = n_o + static_cast<size_t>(obs_chunks(n_spheres));
-  MCP_CUDA(dev_malloc(&ctx->d_obs32, n_rec * 2 * sizeof(float4), "obstacles"), "cudaMalloc obstacles");
+  const size_t n_pair = static_cast<size_t>(obs_pairs(n_spheres) + obs_pairs(obs_chunks(n_spheres)));
+  MCP_CUDA(dev_malloc(&ctx->d_obs32, (n_pair > 0 ? n_pair : 1) * 3 * sizeof(float4), "obstacles"), "cudaMalloc obstacles");
   MCP_CUDA(dev_malloc(&ctx->d_obs64, n_o * 4 * sizeof(double), "obstacles"), "cudaMalloc obstacles");
   MCP_CUDA(dev_malloc(&ctx->d_box32, n_b * 6 * sizeof(float), "boxes"), "cudaMalloc boxes");
   MCP_CUDA(dev_malloc(&ctx->d_box64, n_b * 6 * sizeof(double), "boxes"), "cudaMalloc boxes");

@@ -63,6 +63,8 @@ constexpr int MAXK = 24;
 // chunk of OBS_CHUNK consecutive obstacles (stored in spatial order).
 constexpr int OBS_CHUNK = 16;
 __host__ __device__ constexpr int obs_chunks(int n_obs) { return (n_obs + OBS_CHUNK - 1) / OBS_CHUNK; }
+// Records are kept two to a pair (12 floats).
+__host__ __device__ constexpr int obs_pairs(int n_obs) { return (n_obs + 1) / 2; }
 
 enum : int { REV = 0, PRIS = 1 };
 enum : int {

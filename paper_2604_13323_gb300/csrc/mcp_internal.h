@@ -58,7 +58,7 @@ struct HostModel {
   SphereTable<double> st64;
   const ModelT<double> *d_m64 = nullptr;  // device copy of m64
   const double2 *d_tab = nullptr;         // FP64 sin/cos tables: 256 + 8193 entries
-  const float4 *d_obs32 = nullptr;        // per obstacle 2 x float4: (-2c, |c|^2 - r^2), (-2r, 0, 0, 0), shifted
+  const float4 *d_obs32 = nullptr;        // obstacle and chunk records in pairs (3 x float4 each), shifted
   const double *d_obs64 = nullptr;        // [n_obs * 4]
   const float *d_box32 = nullptr;         // [n_box * 6] lo.xyz, hi.xyz, shifted
   const double *d_box64 = nullptr;        // [n_box * 6]

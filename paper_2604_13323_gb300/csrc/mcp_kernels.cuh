@@ -8,6 +8,7 @@
 // when ||F|| < tol, at the iteration cap, or on a step longer than MaxDistance.
 #pragma once
 
+#include <algorithm>
 #include <cfloat>
 
 #include <math_constants.h>
@@ -984,7 +985,6 @@ struct Rot9 {
 //   A = (gx0, gx1, gy0, gy1), B = (gz0, gz1, gw0, gw1), C = (g20, g21, 0, 0)
 // with g = -2 c, gw = |c|^2 - r^2, g2 = -2 r (the expanded overlap test
 // below).  An odd count is padded with a record that never overlaps.
-__host__ __device__ constexpr int obs_pairs(int n_obs) { return (n_obs + 1) / 2; }
 // The records of the chunk spheres (one per OBS_CHUNK consecutive obstacles,
 // same form) follow the obstacles' pairs, also in pairs: one chunk pair per
 // 32 obstacles.
@@ -1159,26 +1159,16 @@ __device__ __forceinline__ bool check_one_f32(const ModelT<float> &m, const Sphe
   return hit;
 }
 
-// Stages the FP32 obstacle records (in pairs, see obs_rec), the chunk
-// records (in pairs, after them) and the boxes of the collision frame in
-// shared memory: s_pair holds obs_pairs(n_obs) x 3 float4, then
-// obs_pairs(obs_chunks(n_obs)) x 3 float4 of chunks, then the boxes.
-// obs: [(n_obs + obs_chunks(n_obs)) * 8] (gx, gy, gz, gw, g2, 0, 0, 0).
+// Stages the FP32 obstacle records, the chunk records after them (both in
+// pairs, as loaded: 3 float4 each) and the boxes of the collision frame in
+// shared memory: 16-byte copies, the layout having been made when the
+// obstacles were loaded.
 __device__ __forceinline__ float *stage_obstacles(const float *obs, int n_obs, const float *box, int n_box,
                                                   float4 *s_pair) {
-  const int np = obs_pairs(n_obs), nch = obs_chunks(n_obs), ncp = obs_pairs(nch);
-  float *f = reinterpret_cast<float *>(s_pair);
-  for (int t = threadIdx.x; t < 12 * (np + ncp); t += blockDim.x) {
-    const bool chunk = t >= 12 * np;
-    const int u = chunk ? t - 12 * np : t;
-    const int pp = u / 12, c = u % 12, o = 2 * pp + (c & 1), field = c >> 1;  // gx gy gz gw g2 pad
-    const int n = chunk ? nch : n_obs;
-    const float *src = chunk ? obs + 8 * n_obs : obs;
-    float v = 0.f;
-    if (field < 5) v = o < n ? src[8 * o + field] : (field == 3 ? 1e30f : 0.f);  // padding: gw huge
-    f[t] = v;
-  }
-  float *s_box = f + 12 * (np + ncp);
+  const int n4 = 3 * (obs_pairs(n_obs) + obs_pairs(obs_chunks(n_obs)));
+  const float4 *src = reinterpret_cast<const float4 *>(obs);
+  for (int t = threadIdx.x; t < n4; t += blockDim.x) s_pair[t] = __ldg(src + t);
+  float *s_box = reinterpret_cast<float *>(s_pair + n4);
   for (int t = threadIdx.x; t < 6 * n_box; t += blockDim.x) s_box[t] = box[t];
   return s_box;
 }
@@ -1218,6 +1208,82 @@ __global__ void __launch_bounds__(128, (check_min_blocks<P>())) k_check_f32(cons
   const bool hit = check_one_f32<P>(m, a.st, s_pair, a.n_obs, s_box, a.n_box, a.tab, q, tests);
   a.out[i] = hit ? 1 : 0;
   if (a.pairs) a.pairs[i] = tests;
+}
+
+// The same verdict with PARTS lanes per configuration, for batches that leave
+// the SMs idle: every lane places the links (a tenth of one lane's work) and
+// keeps the poses of those dealt to it in shared memory, then the lanes test
+// their k-th links side by side; a configuration is done at its first hit.
+// What bounds it: the latency of one warp's chain, FK and two or three links
+// instead of all.  The lanes must reach the link test together (one call for
+// all of them): testing each link where it is placed runs the links one after
+// the other, with an eighth of the lanes (67 us for 4,099 humanoid
+// configurations; with one lane each 62 us).  The projection and check of
+// those: 346 us with one lane each, 275 us with eight; 8,195 of the arm's
+// bounded TSR 113 us, and 106 us with four.
+template <class P, int PARTS>
+__host__ __device__ constexpr int check_part_links() {  // links (and the world) a lane may be dealt
+  return (P::D + 1 + PARTS - 1) / PARTS;
+}
+template <class P, int PARTS>
+__host__ __device__ constexpr size_t check_part_bytes() {
+  return sizeof(float) * 128 * 13 * check_part_links<P, PARTS>();
+}
+template <class P, int PARTS>
+__global__ void __launch_bounds__(128) k_check_parts(const __grid_constant__ CheckArgs<P, float> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float *pose = reinterpret_cast<float *>(smem_raw) + threadIdx.x;  // entry e of this lane at pose[e * 128]
+  float4 *s_pair = reinterpret_cast<float4 *>(smem_raw + check_part_bytes<P, PARTS>());
+  const float *s_box = stage_obstacles(a.obs, a.n_obs, a.box, a.n_box, s_pair);
+  const long long t = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const long long i = t / PARTS;
+  const int part = static_cast<int>(t) & (PARTS - 1);
+  const bool in = i < a.n;  // lanes past the end only take part in the votes
+  constexpr int D = P::D;
+  int turn = 0, mine = 0;
+  if (in) {
+    float q[D];
+#pragma unroll
+    for (int j = 0; j < D; ++j) q[j] = a.q[j * a.ld + i];
+    const ModelT<float> m = a.m;
+    const OpsF32 ops{a.tab};
+    const auto keep = [&](int link, const float (&R)[9], V3<float> p) {
+      if (a.st.off[link + 1] >= a.st.off[link + 2]) return;
+      if ((turn++ & (PARTS - 1)) == part) {
+        float *o = pose + 128 * 13 * mine++;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) o[128 * e] = R[e];
+        o[128 * 9] = p.x;
+        o[128 * 10] = p.y;
+        o[128 * 11] = p.z;
+        o[128 * 12] = __int_as_float(link);
+      }
+    };
+    const float I[9] = {1.f, 0.f, 0.f, 0.f, 1.f, 0.f, 0.f, 0.f, 1.f};
+    keep(-1, I, V3<float>{-m.shift[0], -m.shift[1], -m.shift[2]});
+    Kin<P, float> k;
+    fk_links<P>(ops, m, q, k, [&](auto JJ, const float (&R)[9], V3<float> p) { keep(decltype(JJ)::value, R, p); }, NoStop{});
+  }
+  __syncthreads();  // the obstacles are staged
+  const int first = (threadIdx.x & 31) & ~(PARTS - 1);
+  const unsigned group = ((1u << PARTS) - 1u) << first;
+  bool hit = false, done = false;
+  for (int k = 0; k < check_part_links<P, PARTS>(); ++k) {
+    const bool test = !done && k < mine;
+    if (!__any_sync(FULL, test)) break;
+    if (test) {
+      const float *o = pose + 128 * 13 * k;
+      Rot9 R;
+#pragma unroll
+      for (int e = 0; e < 9; ++e) R.r[e] = o[128 * e];
+      const int link = __float_as_int(o[128 * 12]);
+      uint32_t tests = 0;
+      hit = link_hits_f32<true>(R, V3<float>{o[128 * 9], o[128 * 10], o[128 * 11]}, a.st.off[link + 1], a.st.off[link + 2],
+                                a.st.lb[link < 0 ? MAXJ : link], a.st, s_pair, a.n_obs, s_box, a.n_box, &tests);
+    }
+    done = (__ballot_sync(FULL, hit) & group) != 0u;
+  }
+  if (in && part == 0) a.out[i] = done ? 1 : 0;
 }
 
 template <class P>
@@ -1931,8 +1997,26 @@ cudaError_t launch_check_impl(const HostModel &hm, const CheckCall &c, int *laun
     a.out = c.out;
     a.pairs = c.pairs;
     a.tab = hm.d_tab;
+    // Lanes per configuration: 8 or 4 while that gives an SM at most 8 warps
+    // (n <= 4,864 and 9,728 on 152 SMs); the count of tests is that of one lane.
     const size_t smem = obs_smem_bytes(hm.n_obs, hm.n_box);
+    const auto parts = [&](auto PP) -> cudaError_t {
+      constexpr int N = decltype(PP)::value;
+      auto kern = k_check_parts<P, N>;
+      const size_t bytes = smem + check_part_bytes<P, N>();
+      if (bytes > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+        if (e != cudaSuccess) return e;
+      }
+      kern<<<static_cast<unsigned>((c.n * N + 127) / 128), 128, bytes, c.stream>>>(a);
+      return cudaGetLastError();
+    };
+    const long long room = 8ll * 32 * hm.sm_count;
+    *launches += 1;
+    if (!c.pairs && P::D >= 7 && c.n * 8 <= room) return parts(std::integral_constant<int, 8>{});
+    if (!c.pairs && P::D >= 7 && c.n * 4 <= room) return parts(std::integral_constant<int, 4>{});
     k_check_f32<P><<<blocks, 128, smem, c.stream>>>(a);
+    return cudaGetLastError();
   }
   *launches += 1;
   return cudaGetLastError();

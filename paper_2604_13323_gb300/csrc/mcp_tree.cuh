@@ -1256,8 +1256,6 @@ cudaError_t launch_project_tree(const HostModel &hm, const ProjCall &c, int *lau
   if (c.precision == 1 || c.segments || c.outer || c.cyclic) return cudaErrorNotSupported;
   if (c.total > 0x7fffffffLL) return cudaErrorInvalidValue;  // parked indices are 32-bit
   TreeArgs<P> a;
-  cudaError_t err = cudaMemsetAsync(c.counter, 0, sizeof(unsigned long long), c.stream);
-  if (err != cudaSuccess) return err;
   a.m = hm.m32;
   a.t = make_tree_const<P>(hm.m32, hm.m64);
   a.m64 = hm.d_m64;
@@ -1285,10 +1283,12 @@ cudaError_t launch_project_tree(const HostModel &hm, const ProjCall &c, int *lau
   if (w > TREE_WARPS) w = TREE_WARPS;
   const size_t smem = tree_smem_bytes<P>(static_cast<int>(w));
   auto kern = k_project_tree<P>;
-  err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (err != cudaSuccess) return err;
   long long blocks = (warps + w - 1) / w;
   if (blocks > hm.sm_count) blocks = hm.sm_count;
+  err = cudaMemsetAsync(c.counter, 0, sizeof(unsigned long long), c.stream);
+  if (err != cudaSuccess) return err;
   kern<<<static_cast<unsigned>(blocks), static_cast<unsigned>(w) * 32, smem, c.stream>>>(a);
   *launches += 1;
   return cudaGetLastError();
