@@ -268,10 +268,11 @@ mcp_status mcp_extend_batch(mcp_ctx *ctx, const mcp_project_params *p, const mcp
  * with ld_out >= sum(len); flags / iters / resid as in mcp_project_batch.
  * The library scans len on the device into context-owned scratch.  Idle
  * lanes refill themselves from a work counter, so segments of any length mix
- * in one launch.  The scan, the counter reset and the projection kernel are
- * captured once into a CUDA graph and replayed while the arguments and the
- * loaded model stay the same (not when the caller's stream is itself being
- * captured: then the kernels are enqueued directly). */
+ * in one launch.  When the same call comes twice in a row (arguments and loaded
+ * model unchanged), the scan, the counter reset and the projection kernel are
+ * captured into a CUDA graph, which is replayed while that call repeats; other
+ * calls, and calls on a stream that is itself being captured, enqueue the
+ * kernels directly. */
 mcp_status mcp_project_segments(mcp_ctx *ctx, const mcp_project_params *p, int64_t n_seg, int64_t ld_seg,
                                 const void *start, const void *delta, const int32_t *len, int64_t total,
                                 int64_t ld_out, void *q_out, uint8_t *flags, uint8_t *iters, double *resid,
@@ -329,7 +330,9 @@ mcp_status mcp_set_tuning(mcp_ctx *ctx, int32_t tpb, int32_t blocks_per_sm, int3
  * fastest in the context for later calls.  With obstacles loaded the timed
  * step is mcp_project_check_batch, and every launch shape is timed with the
  * check inside the projection kernel and as a second launch.  Each candidate
- * is timed as the median of five bursts of four calls.  Uses temporary
+ * is timed as the median of five bursts of four calls; because the choice of
+ * threads per configuration changes results by rounding, one lane per chain is
+ * taken unless one per configuration is faster by more than a quarter.  Uses temporary
  * device buffers; synchronous.  The choices are returned in tpb / blocks_per_sm /
  * chunk / fuse_check / threads_per_config (HOST, each may be NULL).  The
  * launch shape never changes results; threads per configuration changes them
