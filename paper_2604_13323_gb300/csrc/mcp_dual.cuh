@@ -48,15 +48,15 @@ __device__ __forceinline__ float2 pat2_value(float2 v) {
 template <int A>
 __device__ __forceinline__ float2 pat2_fma(float2 v, float2 t, float2 p) {
   if constexpr (A == PZ) return p;
-  else if constexpr (A == PP) return __fadd2_rn(p, t);
+  else if constexpr (A == PP) return add2(p, t);
   else if constexpr (A == PN) return sub2(p, t);
-  else return __ffma2_rn(v, t, p);
+  else return fma2(v, t, p);
 }
 template <int A>
 __device__ __forceinline__ float2 pat2_times(float2 x, float2 nx, float2 v) {  // x v, with nx = -x
   if constexpr (A == PP) return x;
   else if constexpr (A == PN) return nx;
-  else return __fmul2_rn(x, v);
+  else return mul2(x, v);
 }
 template <int A, int B>
 __device__ __forceinline__ void pat2_rotate(float2 c, float2 nc, float2 s, float2 ns, float2 &a, float2 &b) {
@@ -71,8 +71,8 @@ __device__ __forceinline__ void pat2_rotate(float2 c, float2 nc, float2 s, float
     b = pat2_times<B>(c, nc, b0);
   } else {
     static_assert(A == PG && B == PG, "a signed axis stands alone in its row");
-    a = __ffma2_rn(c, a0, __fmul2_rn(s, b0));
-    b = __ffma2_rn(c, b0, __fmul2_rn(ns, a0));
+    a = fma2(c, a0, mul2(s, b0));
+    b = fma2(c, b0, mul2(ns, a0));
   }
 }
 
@@ -257,7 +257,7 @@ __device__ __forceinline__ bool dual_iter_f32(const A &a, float2 *__restrict__ s
 #pragma unroll
       for (int i = 0; i < K; ++i) {
         v[i] = s[i * 32];
-        d = __ffma2_rn(v[i], y2[i], d);
+        d = fma2(v[i], y2[i], d);
       }
       sm[(6 * H + j) * 32] = d;
 #pragma unroll

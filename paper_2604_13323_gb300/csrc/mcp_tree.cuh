@@ -300,16 +300,16 @@ __device__ __forceinline__ void tree_joint2(float2 (&T)[12], const float2 *t, fl
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
     float2 p = T[4 * r + 3];
-    if constexpr (TM & 4) p = __ffma2_rn(T[4 * r + 2], t[2], p);
-    if constexpr (TM & 2) p = __ffma2_rn(T[4 * r + 1], t[1], p);
-    if constexpr (TM & 1) p = __ffma2_rn(T[4 * r], t[0], p);
+    if constexpr (TM & 4) p = fma2(T[4 * r + 2], t[2], p);
+    if constexpr (TM & 2) p = fma2(T[4 * r + 1], t[1], p);
+    if constexpr (TM & 1) p = fma2(T[4 * r], t[0], p);
     const float2 a = T[4 * r + p0], b = T[4 * r + p1], c = T[4 * r + p2];
     if constexpr (p0 < p1) {
-      T[4 * r] = __ffma2_rn(csa, a, __fmul2_rn(snb, b));
-      T[4 * r + 1] = __ffma2_rn(sna, a, __fmul2_rn(csb, b));
+      T[4 * r] = fma2(csa, a, mul2(snb, b));
+      T[4 * r + 1] = fma2(sna, a, mul2(csb, b));
     } else {
-      T[4 * r] = __ffma2_rn(snb, b, __fmul2_rn(csa, a));
-      T[4 * r + 1] = __ffma2_rn(csb, b, __fmul2_rn(sna, a));
+      T[4 * r] = fma2(snb, b, mul2(csa, a));
+      T[4 * r + 1] = fma2(csb, b, mul2(sna, a));
     }
     T[4 * r + 2] = xr_neg(CODE, 2) ? neg2(c) : c;
     T[4 * r + 3] = p;
@@ -326,9 +326,9 @@ __device__ __forceinline__ void tree_frame2(const float2 (&T)[12], const float2 
       R[3 * r + c] = xr_neg(CODE, c) ? neg2(v) : v;
     }
     float2 v = T[4 * r + 3];
-    if constexpr (TM & 4) v = __ffma2_rn(T[4 * r + 2], ft[2], v);
-    if constexpr (TM & 2) v = __ffma2_rn(T[4 * r + 1], ft[1], v);
-    if constexpr (TM & 1) v = __ffma2_rn(T[4 * r], ft[0], v);
+    if constexpr (TM & 4) v = fma2(T[4 * r + 2], ft[2], v);
+    if constexpr (TM & 2) v = fma2(T[4 * r + 1], ft[1], v);
+    if constexpr (TM & 1) v = fma2(T[4 * r], ft[0], v);
     o[r] = v;
   }
   p = V3p{o[0], o[1], o[2]};
@@ -349,9 +349,9 @@ __device__ __forceinline__ V3p tree_limbs(const TreeLimb<N> &m, float2 (&T)[12],
     float2 v[3];
 #pragma unroll
     for (int r = 0; r < 3; ++r)
-      v[r] = __fmul2_rn(m.mass[i], __ffma2_rn(T[4 * r], m.com[i][0],
-                                              __ffma2_rn(T[4 * r + 1], m.com[i][1],
-                                                         __ffma2_rn(T[4 * r + 2], m.com[i][2], T[4 * r + 3]))));
+      v[r] = mul2(m.mass[i], fma2(T[4 * r], m.com[i][0],
+                                              fma2(T[4 * r + 1], m.com[i][1],
+                                                         fma2(T[4 * r + 2], m.com[i][2], T[4 * r + 3]))));
     C[i] = V3p{v[0], v[1], v[2]};
     float2 *s = slot + 8 * 32 * i;
 #pragma unroll
@@ -367,11 +367,11 @@ __device__ __forceinline__ V3p tree_limbs(const TreeLimb<N> &m, float2 (&T)[12],
     // (1/M) z x (C - M_j o), x and y
     const float2 nM = m.nmsub[i];
     const V3p z = load_axis(slot + 8 * 32 * i), o = load_origin(slot + 8 * 32 * i);
-    const V3p rr{__ffma2_rn(nM, o.x, C[i].x), __ffma2_rn(nM, o.y, C[i].y), __ffma2_rn(nM, o.z, C[i].z)};
-    const float2 dx = __ffma2_rn(z.y, rr.z, __fmul2_rn(neg2(z.z), rr.y));
-    const float2 dy = __ffma2_rn(z.z, rr.x, __fmul2_rn(neg2(z.x), rr.z));
-    slot[(8 * i + 6) * 32] = __fmul2_rn(dx, both(inv_mass));
-    slot[(8 * i + 7) * 32] = __fmul2_rn(dy, both(inv_mass));
+    const V3p rr{fma2(nM, o.x, C[i].x), fma2(nM, o.y, C[i].y), fma2(nM, o.z, C[i].z)};
+    const float2 dx = fma2(z.y, rr.z, mul2(neg2(z.z), rr.y));
+    const float2 dy = fma2(z.z, rr.x, mul2(neg2(z.x), rr.z));
+    slot[(8 * i + 6) * 32] = mul2(dx, both(inv_mass));
+    slot[(8 * i + 7) * 32] = mul2(dy, both(inv_mass));
   });
   return C[0];
 }
@@ -505,10 +505,10 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
     ef.x = pf;
 #pragma unroll
     for (int k = 0; k < 3; ++k)
-      ef.x = V3p{__ffma2_rn(Rf[k], a.t.Qp[k], ef.x.x), __ffma2_rn(Rf[3 + k], a.t.Qp[k], ef.x.y),
-                 __ffma2_rn(Rf[6 + k], a.t.Qp[k], ef.x.z)};
+      ef.x = V3p{fma2(Rf[k], a.t.Qp[k], ef.x.x), fma2(Rf[3 + k], a.t.Qp[k], ef.x.y),
+                 fma2(Rf[6 + k], a.t.Qp[k], ef.x.z)};
 #pragma unroll
-    for (int r = 0; r < 3; ++r) tf[r] = __fadd2_rn(row2(a.t.Pr + 3 * r, ef.x), a.t.Pp[r]);
+    for (int r = 0; r < 3; ++r) tf[r] = add2(row2(a.t.Pr + 3 * r, ef.x), a.t.Pp[r]);
     float Pr[9], RaT[9], Rb[9];
     load_R(m.cPinv[2], Pr);
     const V3<float> Pp = load_p(m.cPinv[2]);
@@ -644,9 +644,9 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
 #pragma unroll
   for (int i = 0; i < 3; ++i) ca[i] = cl[i] = make_float2(0.f, 0.f);
   const auto com_add2 = [](float2 (&p)[3], float2 gx, float2 gy) {
-    p[0] = __ffma2_rn(gx, gx, p[0]);
-    p[1] = __ffma2_rn(gy, gx, p[1]);
-    p[2] = __ffma2_rn(gy, gy, p[2]);
+    p[0] = fma2(gx, gx, p[0]);
+    p[1] = fma2(gy, gx, p[1]);
+    p[2] = fma2(gy, gy, p[2]);
   };
   // hands' block and their CoM rows, with the arms' segments built in place
   // (joints above frame a enter with -1, above b with +1): the left arm's
@@ -722,16 +722,16 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
       } else {
         C[i] = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int j = 0; j < 3; ++j) C[i] = __ffma2_rn(both(r == 0 ? jc[j].x : jc[j].y), a.t.jt[j][k < 3 ? k : 0], C[i]);
+        for (int j = 0; j < 3; ++j) C[i] = fma2(both(r == 0 ? jc[j].x : jc[j].y), a.t.jt[j][k < 3 ? k : 0], C[i]);
       }
     }
     const auto add = [&](const float2 (&f)[6], float2 gx, float2 gy) {
 #pragma unroll
       for (int i = 0; i < 6; ++i) {
 #pragma unroll
-        for (int k = 0; k <= i; ++k) B[tri(i, k)] = __ffma2_rn(f[i], f[k], B[tri(i, k)]);
-        C[i] = __ffma2_rn(gx, f[i], C[i]);
-        C[6 + i] = __ffma2_rn(gy, f[i], C[6 + i]);
+        for (int k = 0; k <= i; ++k) B[tri(i, k)] = fma2(f[i], f[k], B[tri(i, k)]);
+        C[i] = fma2(gx, f[i], C[i]);
+        C[6 + i] = fma2(gy, f[i], C[6 + i]);
       }
     };
     float2 Pr[9];
@@ -907,7 +907,7 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
       acc = fmaf(a.t.jt[i][2].y, yf[2].y, acc);
       dqb[i] = com_dot(jc[i], acc);
 #pragma unroll
-      for (int k = 0; k < 3; ++k) rf[k] = __ffma2_rn(a.t.jt[i][k], both(dqb[i]), rf[k]);
+      for (int k = 0; k < 3; ++k) rf[k] = fma2(a.t.jt[i][k], both(dqb[i]), rf[k]);
     }
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
@@ -921,7 +921,7 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
       for (int r = 0; r < 6; r += 2) acc = fmaf(v[r].y, yf[r].y, fmaf(v[r + 1].y, yf[r + 1].y, acc));
       dqb[3 + b] = com_dot(at(TP_BASE + 7 * b + 6), acc);
 #pragma unroll
-      for (int r = 0; r < 6; ++r) rf[r] = __ffma2_rn(v[r], both(dqb[3 + b]), rf[r]);
+      for (int r = 0; r < 6; ++r) rf[r] = fma2(v[r], both(dqb[3 + b]), rf[r]);
     }
     // limbs: the scaled step of the last pass stays in the joint's first slot
     {
@@ -934,14 +934,14 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
         const float2 gx = leg[6 * 32], gy = leg[7 * 32];
         float2 d = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int r = 0; r < 6; r += 2) d = __ffma2_rn(v[r], yf[r], __ffma2_rn(v[r + 1], yf[r + 1], d));
-        d = __ffma2_rn(gx, both(yc[0]), __ffma2_rn(gy, both(yc[1]), d));
-        pl[0] = __ffma2_rn(gx, d, pl[0]);
-        pl[1] = __ffma2_rn(gy, d, pl[1]);
+        for (int r = 0; r < 6; r += 2) d = fma2(v[r], yf[r], fma2(v[r + 1], yf[r + 1], d));
+        d = fma2(gx, both(yc[0]), fma2(gy, both(yc[1]), d));
+        pl[0] = fma2(gx, d, pl[0]);
+        pl[1] = fma2(gy, d, pl[1]);
 #pragma unroll
-        for (int r = 0; r < 6; ++r) rf[r] = __ffma2_rn(v[r], d, rf[r]);
-        const float2 e = __fmul2_rn(d, both(a.alpha));
-        sl = __ffma2_rn(e, e, sl);
+        for (int r = 0; r < 6; ++r) rf[r] = fma2(v[r], d, rf[r]);
+        const float2 e = mul2(d, both(a.alpha));
+        sl = fma2(e, e, sl);
         if (last) leg[0] = e;
       }
     }
