@@ -14,6 +14,8 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>
+
 #include "../../include/mcproj.h"
 #include "mcp_device.cuh"
 #include "mcp_internal.h"
@@ -751,8 +753,31 @@ mcp_status update_shifted(mcp_ctx *ctx) {
   return MCP_OK;
 }
 
+// The driver's query of one attribute (nullptr if it cannot be had): the
+// runtime's cudaPointerGetAttributes asks for all of them, for each of the four
+// to seven pointers of a call.
+decltype(&cuPointerGetAttribute) pointer_attribute() {
+  static const auto fn = [] {
+    void *f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<decltype(&cuPointerGetAttribute)>(f);
+  }();
+  return fn;
+}
+
 mcp_status check_batch_ptr(mcp_ctx *ctx, const void *p, const char *name) {
   if (!p) return fail(ctx, MCP_ERR_ARG, "%s is NULL", name);
+  if (const auto attr = pointer_attribute()) {  // anything but plain device memory is looked at again below
+    CUmemorytype type = static_cast<CUmemorytype>(0);
+    if (attr(&type, CU_POINTER_ATTRIBUTE_MEMORY_TYPE, reinterpret_cast<CUdeviceptr>(p)) == CUDA_SUCCESS &&
+        type == CU_MEMORYTYPE_DEVICE)
+      return MCP_OK;
+  }
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
