@@ -1037,15 +1037,26 @@ static __device__ __noinline__ bool link_hits_f32(const Rot9 Rr, V3<float> p, in
   const float2 bx2 = make_float2(bc.x, bc.x), by2 = make_float2(bc.y, bc.y), bz2 = make_float2(bc.z, bc.z),
                br2 = make_float2(br, br);
   const float4 *s_chunk = s_pair + 3 * obs_pairs(n_obs);
-  // the bounding sphere's 4-FMA test against the records pr[pp] (two per pair)
-  auto pair_bits = [&](const float4 *pr, int pp) -> unsigned {
+  // the bounding sphere's 4-FMA test against the records pr[pp] (two per
+  // pair): v < -kb, i.e. the sign of v + kb (the rounded sum has the sign of
+  // the exact one, and a NaN the GPU makes has its sign clear), shifted into
+  // the mask from below, so that the first record ends up highest.  One packed
+  // addition and two funnel shifts per pair instead of two comparisons, two
+  // selections and two shifted ors (humanoid, 262,147 checks: 327 -> 318 us;
+  // 16,384 extensions 903 -> 890 us)
+  const float2 kb2 = make_float2(kb, kb);
+  auto pair_bits = [&](const float4 *pr, int pp, unsigned m) -> unsigned {
     const float4 A = pr[3 * pp], B = pr[3 * pp + 1], C = pr[3 * pp + 2];
     float2 v = __ffma2_rn(br2, make_float2(C.x, C.y), make_float2(B.z, B.w));
     v = __ffma2_rn(bz2, make_float2(B.x, B.y), v);
     v = __ffma2_rn(by2, make_float2(A.z, A.w), v);
     v = __ffma2_rn(bx2, make_float2(A.x, A.y), v);
-    return (v.x < -kb ? 1u : 0u) | (v.y < -kb ? 2u : 0u);
+    v = __fadd2_rn(v, kb2);
+    m = __funnelshift_l(__float_as_uint(v.x), m, 1);
+    return __funnelshift_l(__float_as_uint(v.y), m, 1);
   };
+  // records k0 .. of a mask of `bits` results, first record at bit k0
+  auto from = [](unsigned m, int bits, int k0) -> unsigned { return (__brev(m) >> (32 - bits)) << k0; };
   for (int o0 = 0; o0 < n_obs && !hit; o0 += 32) {
     const int cnt = min(32, n_obs - o0);
     const float4 *pr = s_pair + 3 * (o0 >> 1);
@@ -1054,29 +1065,35 @@ static __device__ __noinline__ bool link_hits_f32(const Rot9 Rr, V3<float> p, in
       // the two chunks of these 32 obstacles first (a chunk's sphere contains
       // its obstacles, so an obstacle the bound overlaps lies in a chunk it
       // overlaps)
-      const unsigned chunks = pair_bits(s_chunk, o0 >> 5);
+      const unsigned chunks = from(pair_bits(s_chunk, o0 >> 5, 0u), 2, 0);
       tests += cnt > OBS_CHUNK ? 2u : 1u;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         if (!((chunks >> h) & 1u)) continue;
         const int c0 = h * OBS_CHUNK, cc = min(OBS_CHUNK, cnt - c0);
         if (cc <= 0) continue;
-        if (cc == OBS_CHUNK) {  // full chunk: unrolled, compile-time bit positions
+        unsigned m = 0u;
+        if (cc == OBS_CHUNK) {  // full chunk: unrolled
 #pragma unroll
-          for (int pp = 0; pp < OBS_CHUNK / 2; ++pp) cand |= pair_bits(pr, h * (OBS_CHUNK / 2) + pp) << (c0 + 2 * pp);
+          for (int pp = 0; pp < OBS_CHUNK / 2; ++pp) m = pair_bits(pr, h * (OBS_CHUNK / 2) + pp, m);
+          cand |= from(m, OBS_CHUNK, c0);
         } else {  // the padded record of an odd count never overlaps
-          for (int pp = 0; pp < obs_pairs(cc); ++pp) cand |= pair_bits(pr, h * (OBS_CHUNK / 2) + pp) << (c0 + 2 * pp);
+          for (int pp = 0; pp < obs_pairs(cc); ++pp) m = pair_bits(pr, h * (OBS_CHUNK / 2) + pp, m);
+          cand |= from(m, 2 * obs_pairs(cc), c0);
         }
         tests += static_cast<uint32_t>(cc);
       }
     } else {
       // 32 obstacles or fewer: the chunks span the whole scene and rarely
       // prune; every obstacle against the bound
-      if (cnt == 32) {  // full chunk: unrolled, compile-time bit positions
+      unsigned m = 0u;
+      if (cnt == 32) {  // all of them: unrolled
 #pragma unroll
-        for (int pp = 0; pp < 16; ++pp) cand |= pair_bits(pr, pp) << (2 * pp);
+        for (int pp = 0; pp < 16; ++pp) m = pair_bits(pr, pp, m);
+        cand = from(m, 32, 0);
       } else {  // the padded record of an odd count never overlaps
-        for (int pp = 0; pp < obs_pairs(cnt); ++pp) cand |= pair_bits(pr, pp) << (2 * pp);
+        for (int pp = 0; pp < obs_pairs(cnt); ++pp) m = pair_bits(pr, pp, m);
+        cand = from(m, 2 * obs_pairs(cnt), 0);
       }
       tests += static_cast<uint32_t>(cnt);
     }
