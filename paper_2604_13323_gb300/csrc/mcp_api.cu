@@ -452,46 +452,79 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_lengths(const int32_t *le
 }
 
 // Path length and its gradient (thread per waypoint / per path).
+// DIM: the joints at compile time (every load in flight at once, the second
+// pass out of registers; measured with 14 joints and 262,144 waypoints: PATHS),
+// or 0 for any number d, in two passes over memory.
+template <int DIM>
+struct PathRow {  // a column's values, read when needed (DIM = 0) or held
+  float v[DIM > 0 ? DIM : 1];
+  const float *p;
+  long long ld;
+  __device__ __forceinline__ PathRow(const float *q, long long ld_, bool has) : p(has ? q : nullptr), ld(ld_) {
+    if constexpr (DIM > 0) {
+#pragma unroll
+      for (int j = 0; j < DIM; ++j) v[j] = has ? q[j * ld_] : 0.f;
+    }
+  }
+  __device__ __forceinline__ float operator[](int j) const {
+    if constexpr (DIM > 0) return v[j];
+    else return p ? p[j * ld] : 0.f;
+  }
+};
+template <int DIM, class F>
+__device__ __forceinline__ void path_joints(int d, F &&f) {
+  if constexpr (DIM > 0) {
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) f(j);
+  } else {
+    for (int j = 0; j < d; ++j) f(j);
+  }
+}
+
 // One thread per waypoint: d/dq_i of |q_i - q_{i-1}| + |q_{i+1} - q_i|, in two
-// passes over the joints (the norms, then the output; the second pass re-reads
-// the same waypoints from L1) so that nothing is held in runtime-indexed arrays.
+// passes over the joints (the norms, then the output).
+template <int DIM>
 __global__ void k_path_grad(const float *Q, long long ld, long long n_paths, int n_way, int d, float *grad) {
   const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i >= n_paths * n_way) return;
   const int w = static_cast<int>(i % n_way);
   const bool has_p = w > 0, has_n = w + 1 < n_way;
+  const PathRow<DIM> q(Q + i, ld, true), qp(Q + i - 1, ld, has_p), qn(Q + i + 1, ld, has_n);
   float np2 = 0.f, nn2 = 0.f;
-  for (int j = 0; j < d; ++j) {
-    const float qi = Q[j * ld + i];
-    const float ep = has_p ? qi - Q[j * ld + i - 1] : 0.f;
-    const float en = has_n ? Q[j * ld + i + 1] - qi : 0.f;
+  path_joints<DIM>(d, [&](int j) {
+    const float qi = q[j];
+    const float ep = has_p ? qi - qp[j] : 0.f;
+    const float en = has_n ? qn[j] - qi : 0.f;
     np2 = fmaf(ep, ep, np2);
     nn2 = fmaf(en, en, nn2);
-  }
+  });
   const float ip = np2 > 0.f ? rsqrtf(np2) : 0.f;
   const float in = nn2 > 0.f ? rsqrtf(nn2) : 0.f;
-  for (int j = 0; j < d; ++j) {
-    const float qi = Q[j * ld + i];
-    const float ep = has_p ? qi - Q[j * ld + i - 1] : 0.f;
-    const float en = has_n ? Q[j * ld + i + 1] - qi : 0.f;
+  path_joints<DIM>(d, [&](int j) {
+    const float qi = q[j];
+    const float ep = has_p ? qi - qp[j] : 0.f;
+    const float en = has_n ? qn[j] - qi : 0.f;
     grad[j * ld + i] = ep * ip - en * in;
-  }
+  });
 }
 
+template <int DIM>
 __global__ void k_path_step(float *Q, const float *D, long long ld, long long n_paths, int n_way, int d, float eta,
                             float max_step) {
   const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i >= n_paths * n_way) return;
   const int w = static_cast<int>(i % n_way);
   if (w == 0 || w == n_way - 1) return;  // endpoints stay fixed
+  const PathRow<DIM> g(D + i, ld, true), q(Q + i, ld, true);
   float m = 0.f;
-  for (int j = 0; j < d; ++j) m = fmaxf(m, fabsf(eta * D[j * ld + i]));
+  path_joints<DIM>(d, [&](int j) { m = fmaxf(m, fabsf(eta * g[j])); });
   const float sc = (max_step > 0.f && m > max_step) ? max_step / m : 1.f;
-  for (int j = 0; j < d; ++j) Q[j * ld + i] = fmaf(-sc * eta, D[j * ld + i], Q[j * ld + i]);
+  path_joints<DIM>(d, [&](int j) { Q[j * ld + i] = fmaf(-sc * eta, g[j], q[j]); });
 }
 
 // One warp per path: lane l sums the lengths of segments l, l + 32, ... and
 // the warp adds the partial sums in a fixed order (deterministic).
+template <int DIM>
 __global__ void k_path_length(const float *Q, long long ld, long long n_paths, int n_way, int d, float *length) {
   const long long p = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -499,16 +532,24 @@ __global__ void k_path_length(const float *Q, long long ld, long long n_paths, i
   float L = 0.f;
   for (int w = lane; w + 1 < n_way; w += 32) {
     const long long i = p * n_way + w;
+    const PathRow<DIM> q(Q + i, ld, true), qn(Q + i + 1, ld, true);
     float n2 = 0.f;
-    for (int j = 0; j < d; ++j) {
-      const float e = Q[j * ld + i + 1] - Q[j * ld + i];
+    path_joints<DIM>(d, [&](int j) {
+      const float e = qn[j] - q[j];
       n2 = fmaf(e, e, n2);
-    }
+    });
     L += sqrtf(n2);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
   if (lane == 0) length[p] = L;
+}
+// The path kernels of the arms' joint counts are compiled for them.
+template <class F>
+static void with_path_dim(int d, F &&f) {
+  if (d == 14) f(std::integral_constant<int, 14>{});
+  else if (d == 7) f(std::integral_constant<int, 7>{});
+  else f(std::integral_constant<int, 0>{});
 }
 
 // Arithmetic-throughput probe: every thread advances 8 independent FMA
@@ -1588,12 +1629,17 @@ mcp_status mcp_path_length_grad(mcp_ctx *ctx, int64_t n_paths, int32_t n_way, in
   const int d = ctx->robot.nj;
   if (grad) {
     const long long n = n_paths * n_way;
-    k_path_grad<<<static_cast<unsigned>((n + 127) / 128), 128, 0, s>>>(Q, ld, n_paths, n_way, d, grad);
+    with_path_dim(d, [&](auto DD) {
+      k_path_grad<decltype(DD)::value><<<static_cast<unsigned>((n + 127) / 128), 128, 0, s>>>(Q, ld, n_paths, n_way, d, grad);
+    });
     ctx->launches += 1;
     MCP_CUDA(cudaGetLastError(), "path gradient launch");
   }
   if (length) {
-    k_path_length<<<static_cast<unsigned>((n_paths * 32 + 127) / 128), 128, 0, s>>>(Q, ld, n_paths, n_way, d, length);
+    with_path_dim(d, [&](auto DD) {
+      k_path_length<decltype(DD)::value>
+          <<<static_cast<unsigned>((n_paths * 32 + 127) / 128), 128, 0, s>>>(Q, ld, n_paths, n_way, d, length);
+    });
     ctx->launches += 1;
     MCP_CUDA(cudaGetLastError(), "path length launch");
   }
@@ -1635,8 +1681,11 @@ mcp_status mcp_path_step(mcp_ctx *ctx, int64_t n_paths, int32_t n_way, int64_t l
   if ((st = check_batch_ptr(ctx, D, "D")) != MCP_OK) return st;
   DeviceGuard gd(ctx->device);
   const long long n = n_paths * n_way;
-  k_path_step<<<static_cast<unsigned>((n + 127) / 128), 128, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-      Q, D, ld, n_paths, n_way, ctx->robot.nj, eta, max_step);
+  with_path_dim(ctx->robot.nj, [&](auto DD) {
+    k_path_step<decltype(DD)::value>
+        <<<static_cast<unsigned>((n + 127) / 128), 128, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
+            Q, D, ld, n_paths, n_way, ctx->robot.nj, eta, max_step);
+  });
   ctx->launches += 1;
   MCP_CUDA(cudaGetLastError(), "path step launch");
   return MCP_OK;
