@@ -49,9 +49,7 @@ UNIT = "projections/s"
 # dominant kernel, from one ncu capture of the kernel built from this source
 # (profiles/ gives the command and the full capture summary).  Keyed by
 # (workload, kernel); an entry is removed whenever its kernel changes.
-MEASURED_TRAFFIC = {
-    ("arm7_axis_65536", "k_project_f32+check"): 2003456,                  # read 2.00 MB, write 0
-}
+MEASURED_TRAFFIC = {}
 L2_FLUSH_BYTES = 512 << 20   # > 129 MB L2
 
 

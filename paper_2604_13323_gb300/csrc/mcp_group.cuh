@@ -483,7 +483,7 @@ struct __align__(16) GrpState {
   static_assert(LC >= K2, "y and dq must not overlap the Gram matrix");
 };
 
-// Model data the group kernel reads with runtime joint indices (shared memory).
+// Model data read with runtime joint indices (shared memory).
 template <class P>
 struct GrpTables {
   float X[P::D][12];

@@ -10,8 +10,8 @@
 // code of more than the instruction cache holds; a scheduler has two warps.
 // (Four lanes per configuration, with the Jacobian, Gram matrix and factor in
 // shared memory, took 16,000 warp-instructions per iteration for 8
-// configurations: 20.7 ms for 1,048,576 configurations, 667 us for 4,099 and
-// 410 us for 32, against 6.2 ms, 270 us and 140 us here.)  Layout:
+// configurations.  Projection and check of 1,048,576 configurations 21.9 ms,
+// of 4,099 744 us, of 32 410 us; here 7.3 ms, 275 us and 140 us.)  Layout:
 //   * shared memory per configuration: 129 float2 (TREE_PAIRS), lane-major
 //     (pair e of lane l at [e * 32 + l]: conflict-free 64-bit accesses at
 //     immediate offsets); seven warps of 32 configurations fill an SM's 227 KB;
@@ -96,7 +96,7 @@ __host__ __device__ constexpr bool tree_layout_matches() {
 // (the left arm 0, the right arm 1, the left leg and the neck 2, the right leg
 // 3), the trunk spread over them.  Within a partial the limb joints come
 // first, in ascending order, then the trunk's.  This is the dq partition of
-// the group kernel's work plan.
+// the work plan.
 __host__ __device__ constexpr int tree_part(int j) {
   if (j >= TR_ARM0) return j < TR_ARM0 + TR_ARM ? 0 : 1;
   if (j >= TR_NECK) return 2;
