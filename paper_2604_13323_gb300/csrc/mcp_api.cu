@@ -545,6 +545,7 @@ __global__ void k_path_length(const float *Q, long long ld, long long n_paths, i
   for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
   if (lane == 0) length[p] = L;
 }
+
 // The path kernels of the arms' joint counts are compiled for them.
 template <class F>
 static void with_path_dim(int d, F &&f) {
