@@ -866,11 +866,13 @@ __device__ __noinline__ double finish_f64(const A &a, float *q, double *qd, int 
 // Acceptance of one configuration that left the FP32 loop: the FP32 iterate
 // is re-checked with the FP64 residual.  If the FP32 test was too optimistic
 // and steps remain, the configuration goes back to the FP32 loop for one more
-// step (retry allowed: returns true, nothing written); otherwise, or when the
-// FP32 pivot was too small, finish_f64 takes the remaining steps in FP64.
-// Writes q (if changed), flags, iters and resid.
+// step (returns true, nothing written); otherwise, or when the FP32 pivot was
+// too small, finish_f64 takes the remaining steps in FP64.  Which of these is
+// decided by the configuration alone: the callers accept no more of them than
+// they could send back, so that a result does not depend on what else a warp
+// happens to hold.  Writes q (if changed), flags, iters and resid.
 template <class P, int FORM, class A>
-__device__ __forceinline__ bool accept_one(const A &a, long long item, int it, uint32_t fl, bool retry_ok = false) {
+__device__ __forceinline__ bool accept_one(const A &a, long long item, int it, uint32_t fl) {
   constexpr int D = P::D;
   const ModelT<double> &m = *a.m64;
   float q[D];
@@ -878,7 +880,7 @@ __device__ __forceinline__ bool accept_one(const A &a, long long item, int it, u
 #pragma unroll
   for (int j = 0; j < D; ++j) q[j] = ok ? a.q_out[j * a.ld_out + item] : 0.f;
   double r2 = residual2_f64<P>(OpsF64Split{a.tab}, m, q);
-  if (retry_ok && (fl & FL_INT_FP32CONV) && !(r2 < a.tol2_64) && r2 <= DBL_MAX && it < a.cap) return true;
+  if ((fl & FL_INT_FP32CONV) && !(r2 < a.tol2_64) && r2 <= DBL_MAX && it < a.cap) return true;
   if (fl & (FL_INT_FP32CONV | FL_INT_NEEDS_F64)) {
     const bool was_conv = (fl & FL_INT_FP32CONV) != 0;
     fl &= ~(FL_INT_FP32CONV | FL_INT_NEEDS_F64);
@@ -1365,7 +1367,12 @@ __host__ __device__ constexpr int min_blocks() {
 }
 
 // Configurations a warp can hold for an FP32 retry after a failed FP64
-// acceptance (beyond this the acceptance finishes them in FP64 itself).
+// acceptance.  A warp accepts at most as many as still fit (RETRY_CAP - nret),
+// and fills idle lanes only while fewer than 32 are parked: new work is claimed
+// when every retry has found a lane, so that a warp then holds its lanes and at
+// most 31 parked configurations, and, as nothing else adds to them, never more
+// than 63 (positions of s_item).  With 32 or more parked, at most 31 retries are
+// therefore waiting, and at least one can be accepted.
 constexpr int RETRY_CAP = 32;
 
 // Bytes of the Newton step's slots in shared memory (classes whose stacked
@@ -1411,7 +1418,7 @@ __global__ void __launch_bounds__(TPB, (min_blocks<P, TPB, FORM>())) k_project_f
 
   while (true) {
     // (1) refill: configurations sent back by the acceptance first, then new work
-    const unsigned idle = __ballot_sync(FULL, !act);
+    const unsigned idle = __ballot_sync(FULL, !act && pend < 32);
     if (idle != 0u && (nret > 0 || qn < qe || more)) {
       const int n_idle = __popc(idle);
       const int from_r = n_idle < nret ? n_idle : nret;
@@ -1493,8 +1500,7 @@ __global__ void __launch_bounds__(TPB, (min_blocks<P, TPB, FORM>())) k_project_f
     // a failed acceptance with steps left is queued for one more FP32 step
     // (an FP64 step on one lane would hold the FP64 pipe as long as 32 lanes)
     if (pend >= 32 || (drained && pend > 0)) {
-      const int take = pend < 32 ? pend : 32;
-      const bool room = nret + take <= RETRY_CAP;
+      const int take = min(min(pend, 32), RETRY_CAP - nret);
       bool retry = false;
       long long it_item = 0;
       uint32_t meta = 0;
@@ -1502,7 +1508,7 @@ __global__ void __launch_bounds__(TPB, (min_blocks<P, TPB, FORM>())) k_project_f
         const int pos = pend - take + lane;
         meta = s_meta[wib][pos];
         it_item = s_item[wib][pos];
-        retry = accept_one<P, FORM>(a, it_item, static_cast<int>(meta & 0xffu), meta >> 8, room);
+        retry = accept_one<P, FORM>(a, it_item, static_cast<int>(meta & 0xffu), meta >> 8);
         if constexpr (CHK) {
           if (!retry) {
             float qc[D];

@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(TPB, (pair_min_blocks<TPB>())) k_project_pair(
 
   while (true) {
     // (1) refill idle pairs: retries first, then new work
-    const unsigned idle = __ballot_sync(FULL, !act) & EVEN;
+    const unsigned idle = __ballot_sync(FULL, !act && pend < 32) & EVEN;
     if (idle != 0u && (nret > 0 || qn < qe || more)) {
       const int n_idle = __popc(idle);
       const int from_r = n_idle < nret ? n_idle : nret;
@@ -333,8 +333,7 @@ __global__ void __launch_bounds__(TPB, (pair_min_blocks<TPB>())) k_project_pair(
     // (4) FP64 acceptance, one configuration per lane; a failed acceptance
     // with steps left goes back to the FP32 loop
     if (pend >= 32 || (drained && pend > 0)) {
-      const int take = pend < 32 ? pend : 32;
-      const bool room = nret + take <= RETRY_CAP;
+      const int take = min(min(pend, 32), RETRY_CAP - nret);
       bool retry = false;
       long long it_item = 0;
       uint32_t meta = 0;
@@ -342,7 +341,7 @@ __global__ void __launch_bounds__(TPB, (pair_min_blocks<TPB>())) k_project_pair(
         const int pos = pend - take + lane;
         meta = s_meta[wib][pos];
         it_item = s_item[wib][pos];
-        retry = accept_one<P, FORM_STACKED>(a, it_item, static_cast<int>(meta & 0xffu), meta >> 8, room);
+        retry = accept_one<P, FORM_STACKED>(a, it_item, static_cast<int>(meta & 0xffu), meta >> 8);
         if constexpr (CHK) {  // the collision check of the accepted output, one configuration per lane
           if (!retry) {
             float qc[P::D];

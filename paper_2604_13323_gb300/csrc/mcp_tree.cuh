@@ -1056,6 +1056,13 @@ __device__ __forceinline__ bool tree_iter(const A &a, const TreeTeam team, float
 // per lane).  A 32-word scratch per warp routes them.  An acceptance always
 // runs once a warp could not hold another iteration's 32 configurations, or
 // the team has nothing else to do, with or without the token.
+// Whether a failed acceptance goes back is decided by the configuration alone
+// (never by what the warp holds at that moment, which depends on the other
+// warps): a warp accepts no more than still fit among its retries, and fills
+// idle lanes only with at most 64 parked.  New work is claimed when every retry
+// has found a lane; the warp then holds its lanes and at most 64 parked, and as
+// nothing else adds to them, never more than 96.  With more than 64 parked, at
+// most 31 retries are therefore waiting, and an acceptance can go on.
 constexpr int TREE_WARPS = 7;
 constexpr int TREE_TEAM = 4;
 constexpr int TREE_ACCEPT_MIN = 20;
@@ -1093,7 +1100,7 @@ __global__ void __launch_bounds__(TREE_WARPS * 32, 1) k_project_tree(const __gri
   for (int j = 0; j < D; ++j) q[j] = 0.f;
   while (true) {
     // refill idle lanes: retries first, then new work
-    const unsigned idle = __ballot_sync(FULL, !act);
+    const unsigned idle = __ballot_sync(FULL, !act && pend <= 32 * (TREE_SLOTS - 1));
     if (idle != 0u && (nret > 0 || qn < qe || an < ae || more)) {
       const int n_idle = __popc(idle);
       const int from_r = n_idle < nret ? n_idle : nret;
@@ -1213,9 +1220,8 @@ __global__ void __launch_bounds__(TREE_WARPS * 32, 1) k_project_tree(const __gri
       if (wib == team0 && lane == 0) token = atomicCAS(&fp64_taken, 0, 1) == 0;
       accept = full || team.any(token || drained);
     }
-    if (accept && pend > 0 && (pend >= TREE_ACCEPT_MIN || drained)) {
-      const int take = pend < 32 ? pend : 32;
-      const bool room = nret + take <= 32;
+    const int take = min(min(pend, 32), 32 - nret);  // as many as could all be sent back
+    if (accept && take > 0 && (take >= TREE_ACCEPT_MIN || drained || pend > 32 * (TREE_SLOTS - 1))) {
       const int pos = pend - take + lane;
       int it_item = 0, im = 0;
 #pragma unroll
@@ -1228,7 +1234,7 @@ __global__ void __launch_bounds__(TREE_WARPS * 32, 1) k_project_tree(const __gri
       }
       const uint32_t meta = static_cast<uint32_t>(im);
       bool retry = false;
-      if (lane < take) retry = accept_one<P, FORM_STACKED>(a, it_item, static_cast<int>(meta & 0xffu), meta >> 8, room);
+      if (lane < take) retry = accept_one<P, FORM_STACKED>(a, it_item, static_cast<int>(meta & 0xffu), meta >> 8);
       const unsigned rmask = __ballot_sync(FULL, retry);
       if (rmask != 0u) {
         const int nr = __popc(rmask), rank = __popc(rmask & ((1u << lane) - 1u)), s0 = lane - nret;

@@ -765,7 +765,8 @@ __global__ void __launch_bounds__(W * 32, 512 / (W * 32)) k_project_warp(const _
     }
     const bool drained = !have && !more;  // (no retry pending either)
     if (pend == 32 || (drained && pend > 0)) {
-      const bool room = nret + pend <= RETRY_CAP;
+      // every retry was taken up before new work, so that pend + nret <= 32 and
+      // as many as fail fit into the list
       bool retry = false;
       long long it_item = 0;
       uint32_t meta = 0;
@@ -773,7 +774,7 @@ __global__ void __launch_bounds__(W * 32, 512 / (W * 32)) k_project_warp(const _
         meta = s_meta[wib][lane];
         it_item = s_item[wib][lane];
         retry = accept_one<P, CYC ? FORM_CYCLIC : FORM_STACKED>(a, it_item, static_cast<int>(meta & 0xffu),
-                                                                meta >> 8, room);
+                                                                meta >> 8);
       }
       const unsigned rm = __ballot_sync(FULL, retry);
       __syncwarp();
