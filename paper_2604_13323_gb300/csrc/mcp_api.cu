@@ -1116,6 +1116,7 @@ mcp_status mcp_get_constraint(const mcp_ctx *ctx, int32_t i, double *P, double *
 mcp_status mcp_load_obstacles(mcp_ctx *ctx, const double *spheres, int32_t n_spheres, const double *aabbs,
                               int32_t n_aabbs) {
   if (!ctx) return MCP_ERR_ARG;
+  static_assert(MCP_MAX_OBSTACLES == MAXOBS && MCP_MAX_AABBS == MAXBOX, "shared memory of the checks is sized by these");
   if (n_spheres < 0 || n_spheres > MCP_MAX_OBSTACLES || n_aabbs < 0 || n_aabbs > MCP_MAX_AABBS)
     return fail(ctx, MCP_ERR_ARG, "obstacle counts %d / %d outside [0, %d] / [0, %d]", n_spheres, n_aabbs,
                 MCP_MAX_OBSTACLES, MCP_MAX_AABBS);

@@ -59,6 +59,8 @@ constexpr int MAXJ = 40;
 constexpr int MAXF = 8;
 constexpr int MAXC = 8;
 constexpr int MAXK = 24;
+constexpr int MAXOBS = 1024;
+constexpr int MAXBOX = 64;
 // The collision check's broad phase first tests a bounding sphere of each
 // chunk of OBS_CHUNK consecutive obstacles (stored in spatial order).
 constexpr int OBS_CHUNK = 16;

@@ -398,9 +398,10 @@ template <class P, int G>
 cudaError_t launch_extend_g(const HostModel &hm, const ExtCall &c, ExtArgs<P> &a, int *launches) {
   constexpr int W = 2;
   auto kern = k_extend<P, W, G>;
-  const size_t smem = obs_smem_bytes(hm.n_obs, hm.n_box) + static_cast<size_t>(W) * 32 * iter_smem<P, FORM_STACKED>();
+  constexpr size_t slots = static_cast<size_t>(W) * 32 * iter_smem<P, FORM_STACKED>();
+  const size_t smem = obs_smem_bytes(hm.n_obs, hm.n_box) + slots;
   cudaError_t err = cudaSuccess;
-  if (smem > 48 * 1024) err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (smem > 48 * 1024) err = allow_smem(kern, OBS_SMEM_MAX + slots);
   if (err != cudaSuccess) return err;
   int per_sm = 0;
   err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, W * 32, smem);

@@ -994,6 +994,16 @@ __host__ __device__ constexpr size_t obs_smem_bytes(int n_obs, int n_box) {
   return sizeof(float) * (12 * static_cast<size_t>(obs_pairs(n_obs)) + 12 * static_cast<size_t>(obs_pairs(obs_chunks(n_obs))) +
                           6 * static_cast<size_t>(n_box));
 }
+// Lets a kernel take `most` bytes of dynamic shared memory.  The limit belongs
+// to the kernel, for every context and host thread of the process: it is always
+// set to the most that any call of this kernel may need, never to what the
+// present call needs, so that no call lowers it between another thread's call
+// of this and its launch.
+constexpr size_t OBS_SMEM_MAX = obs_smem_bytes(MAXOBS, MAXBOX);
+template <class K>
+cudaError_t allow_smem(K kern, size_t most) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most));
+}
 // Obstacle o's five values from its pair.
 struct ObsRec {
   float gx, gy, gz, gw, g2;
@@ -1872,8 +1882,8 @@ cudaError_t launch_persistent(const HostModel &hm, const ProjCall &c, const Src 
   a.pairs = c.pairs;
   const size_t smem = (CHK ? obs_smem_bytes(hm.n_obs, hm.n_box) : 0) + static_cast<size_t>(TPB) * iter_smem<P, FORM>();
   auto kern = k_project_f32<P, Src, TPB, FORM, CHK>;
-  if (smem > 40 * 1024) {  // with the kernel's static arrays above the 48 KB a launch gets unasked
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (smem > 36 * 1024) {  // with the kernel's static arrays above the 48 KB a launch gets unasked
+    const cudaError_t e = allow_smem(kern, (CHK ? OBS_SMEM_MAX : 0) + static_cast<size_t>(TPB) * iter_smem<P, FORM>());
     if (e != cudaSuccess) return e;
   }
   const long long warps_needed = (c.total + 31) / 32;
@@ -2028,7 +2038,7 @@ cudaError_t launch_check_impl(const HostModel &hm, const CheckCall &c, int *laun
       auto kern = k_check_parts<P, N>;
       const size_t bytes = smem + check_part_bytes<P, N>();
       if (bytes > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+        const cudaError_t e = allow_smem(kern, OBS_SMEM_MAX + check_part_bytes<P, N>());
         if (e != cudaSuccess) return e;
       }
       kern<<<static_cast<unsigned>((c.n * N + 127) / 128), 128, bytes, c.stream>>>(a);

@@ -1289,7 +1289,7 @@ cudaError_t launch_project_tree(const HostModel &hm, const ProjCall &c, int *lau
   if (w > TREE_WARPS) w = TREE_WARPS;
   const size_t smem = tree_smem_bytes<P>(static_cast<int>(w));
   auto kern = k_project_tree<P>;
-  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t err = allow_smem(kern, tree_smem_bytes<P>(TREE_WARPS));
   if (err != cudaSuccess) return err;
   long long blocks = (warps + w - 1) / w;
   if (blocks > hm.sm_count) blocks = hm.sm_count;
