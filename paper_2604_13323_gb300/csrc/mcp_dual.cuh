@@ -3,9 +3,10 @@
 // chains in every instruction.
 //
 // What bounds it: instruction fetch.  Unrolled for one configuration in
-// registers the step was 2,900 instructions (46 KB): with 11 unsynchronised
-// warps on an SM two thirds of their time went to waiting for instructions
-// (5.9 of 8 cycles per issue, 0.27 instructions per cycle and scheduler).
+// registers the step is 2,900 instructions (46 KB): with 11 unsynchronised
+// warps on an SM two thirds of their time go to waiting for instructions
+// (5.9 of 8 cycles per issue, 0.27 instructions per cycle and scheduler).  With
+// fewer warps on an SM that step is still the faster one (dual_in_registers).
 // Here the chains are the two halves of packed FP32x2 operations
 // (mcp_pack.cuh), the Jacobian lives in shared memory (49 float2 per lane,
 // lane-major) and is built and used in loops over the chain's joints: about

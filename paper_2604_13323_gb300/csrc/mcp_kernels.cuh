@@ -23,8 +23,10 @@ namespace mcp {
 
 // Forms of getDescentStep (Alg. 2): the stacked inner step J^T (J J^T + lambda I)^-1 F,
 // one inner step per constraint in turn (cyclic), or the stacked outer step
-// (J^T J + lambda I)^-1 J^T F (a d x d system).
-enum : int { FORM_STACKED = 0, FORM_CYCLIC = 1, FORM_OUTER = 2 };
+// (J^T J + lambda I)^-1 J^T F (a d x d system).  FORM_STACKED_REGS is the stacked
+// step of the dual arm held in registers (newton_iter_f32) instead of shared
+// memory (dual_iter_f32): the same bits, see dual_in_registers.
+enum : int { FORM_STACKED = 0, FORM_CYCLIC = 1, FORM_OUTER = 2, FORM_STACKED_REGS = 3 };
 
 // ---------------------------------------------------------------------------
 // Stacked residual F(q) and Jacobian J(q)
@@ -1947,6 +1949,24 @@ cudaError_t check_outputs(const HostModel &hm, const ProjCall &c, int *launches)
   return launch_check_impl<P>(hm, cc, launches);
 }
 
+// Whether the dual arm's step runs out of registers.  With no more than 12 warps
+// on an SM (what 168 registers a thread allow) its 2,900 unrolled instructions
+// are fetched for few enough warps that the latency of one configuration
+// decides, and there they are ahead of the 2,000 of the looped step with its
+// shared-memory accesses; above, the looped step and its 16 warps.  Times in
+// us, shared memory and registers, default shape: projection of 257 61.2 /
+// 50.8, 16,384 83.7 / 74.6, 48,640 132 / 109, 58,368 139 / 122, 65,536 143 /
+// 150, 262,144 389 / 411; segments of 5,000 points 110 / 92, 32,000 150 / 141,
+// 54,000 167 / 159, 60,000 179 / 205, 262,144 521 / 631.  A launch shape of few
+// warps: batch of 262,144 at 128 x 1 835 / 686, at 256 x 1 617 / 547; segments
+// of 262,144 points 979 / 1,009 and 682 / 726, so there the number of points
+// alone decides.
+inline bool dual_in_registers(const HostModel &hm, const ProjCall &c, int tpb) {
+  long long warps = (c.total + 31) / 32;
+  if (!c.segments) warps = std::min(warps, static_cast<long long>(hm.sm_count) * c.tune.blocks_per_sm * (tpb / 32));
+  return warps <= 12ll * hm.sm_count;
+}
+
 template <class P>
 cudaError_t launch_project_impl(const HostModel &hm, const ProjCall &c, int *launches) {
   if (c.total <= 0) return cudaSuccess;
@@ -1976,10 +1996,16 @@ cudaError_t launch_project_impl(const HostModel &hm, const ProjCall &c, int *lau
     if constexpr (P::NC > 1) {  // one constraint: the cyclic and stacked forms coincide
       if (c.cyclic) return launch_persistent<P, S, 128, FORM_CYCLIC, CHK>(hm, c, src);
     }
+    const auto stacked = [&](auto TT) -> cudaError_t {
+      constexpr int TPB = decltype(TT)::value;
+      if constexpr (dual_layout_matches<P>())
+        if (dual_in_registers(hm, c, TPB)) return launch_persistent<P, S, TPB, FORM_STACKED_REGS, CHK>(hm, c, src);
+      return launch_persistent<P, S, TPB, FORM_STACKED, CHK>(hm, c, src);
+    };
     switch (c.tune.tpb) {
-      case 64: return launch_persistent<P, S, 64, FORM_STACKED, CHK>(hm, c, src);
-      case 256: return launch_persistent<P, S, 256, FORM_STACKED, CHK>(hm, c, src);
-      default: return launch_persistent<P, S, 128, FORM_STACKED, CHK>(hm, c, src);
+      case 64: return stacked(std::integral_constant<int, 64>{});
+      case 256: return stacked(std::integral_constant<int, 256>{});
+      default: return stacked(std::integral_constant<int, 128>{});
     }
   };
   if (c.segments) {
