@@ -1249,9 +1249,8 @@ __global__ void __launch_bounds__(128, (check_min_blocks<P>())) k_check_f32(cons
 // instead of all.  The lanes must reach the link test together (one call for
 // all of them): testing each link where it is placed runs the links one after
 // the other, with an eighth of the lanes (67 us for 4,099 humanoid
-// configurations; with one lane each 62 us).  The projection and check of
-// those: 346 us with one lane each, 275 us with eight; 8,195 of the arm's
-// bounded TSR 113 us, and 106 us with four.
+// configurations; with one lane each 62 us, with eight 21 us).  Where more
+// lanes stop paying is written at the rule (launch_check_impl).
 template <class P, int PARTS>
 __host__ __device__ constexpr int check_part_links() {  // links (and the world) a lane may be dealt
   return (P::D + 1 + PARTS - 1) / PARTS;
@@ -2056,8 +2055,18 @@ cudaError_t launch_check_impl(const HostModel &hm, const CheckCall &c, int *laun
     a.out = c.out;
     a.pairs = c.pairs;
     a.tab = hm.d_tab;
-    // Lanes per configuration: 8 or 4 while that gives an SM at most 8 warps
-    // (n <= 4,864 and 9,728 on 152 SMs); the count of tests is that of one lane.
+    // Lanes per configuration: 8 while that gives an SM at most 16 warps (n <=
+    // 9,728 on 152 SMs) and no more than its shared memory holds at once, 4 while
+    // at most 20 (n <= 24,320); the count of tests is that of one lane.  Times in us with 1 / 4 / 8 lanes: 512 configurations of
+    // the arm 14.7 / 8.6 / 6.7, the dual arm 25.0 / 14.6 / 10.7, the humanoid
+    // 68.1 / 27.1 / 20.8; 9,728: 14.6 / 10.5 / 10.3, 25.0 / 16.8 / 16.7, 72.1 /
+    // 32.6 / 29.0 (the arm's bounded TSR 10.6 / 8.4 / 7.0); 14,592: 14.6 / 10.7 /
+    // 13.5, 25.1 / 18.8 / 24.4, 72.1 / 35.2 / 46.0; 24,320: 16.7 / 12.8 / 16.7,
+    // 29.2 / 26.2 / 31.4, 80.4 / 63.9 / 63.9 (TSR 10.7 / 8.6 / 10.7); 29,184:
+    // 16.7 / 17.0 / 18.9, 29.1 / 33.3 / 37.7, 84.4 / 66.3 / 78.5 (TSR 10.9 / 11.4 /
+    // 12.7).  With 1,000 obstacles (blocks of 61 and 94 KB) the humanoid's 7,296
+    // 203 / 80 / 64, 9,728 207 / 80 / 107, 24,320 232 / 216 / 207; with 4, 24,320
+    // 18.7 / 18.9 / 22.8.
     const size_t smem = obs_smem_bytes(hm.n_obs, hm.n_box);
     const auto parts = [&](auto PP) -> cudaError_t {
       constexpr int N = decltype(PP)::value;
@@ -2070,10 +2079,12 @@ cudaError_t launch_check_impl(const HostModel &hm, const CheckCall &c, int *laun
       kern<<<static_cast<unsigned>((c.n * N + 127) / 128), 128, bytes, c.stream>>>(a);
       return cudaGetLastError();
     };
-    const long long room = 8ll * 32 * hm.sm_count;
+    const auto warps_per_sm = [&](int lanes) { return (c.n * lanes + 32ll * hm.sm_count - 1) / (32ll * hm.sm_count); };
+    constexpr size_t SM_SMEM = 228 * 1024, BLOCK_SMEM = 1024;  // of an SM; what a block takes besides its own
+    const long long held = 4 * static_cast<long long>(SM_SMEM / (smem + check_part_bytes<P, 8>() + BLOCK_SMEM));
     *launches += 1;
-    if (!c.pairs && P::D >= 7 && c.n * 8 <= room) return parts(std::integral_constant<int, 8>{});
-    if (!c.pairs && P::D >= 7 && c.n * 4 <= room) return parts(std::integral_constant<int, 4>{});
+    if (!c.pairs && P::D >= 7 && warps_per_sm(8) <= std::min(16ll, held)) return parts(std::integral_constant<int, 8>{});
+    if (!c.pairs && P::D >= 7 && warps_per_sm(4) <= 20) return parts(std::integral_constant<int, 4>{});
     k_check_f32<P><<<blocks, 128, smem, c.stream>>>(a);
     return cudaGetLastError();
   }

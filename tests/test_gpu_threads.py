@@ -43,7 +43,7 @@ def _calls(mcproj, name):
             out.append(lambda P=P, q=q, s=None: P.project(q, wl.params, stream=s))
         return out
     if name == "check":      # four lanes per configuration: 66 KB and the scene
-        n = 8 * 32 * torch.cuda.get_device_properties(0).multi_processor_count // 8 + 1
+        n = 16 * 32 * torch.cuda.get_device_properties(0).multi_processor_count // 8 + 1
         wl = W.humanoid_workload(n=n)
         out = []
         for k in (8, 1000):
