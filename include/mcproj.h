@@ -327,12 +327,15 @@ mcp_status mcp_set_tuning(mcp_ctx *ctx, int32_t tpb, int32_t blocks_per_sm, int3
  * threads per configuration where the class has a choice) for
  * the loaded problem by timing every candidate on the caller's sample
  * q_sample (DEVICE, float [d * ld], n_sample configurations), and keeps the
- * fastest in the context for later calls.  With obstacles loaded the timed
+ * fastest shape in the context for later calls.  With obstacles loaded the timed
  * step is mcp_project_check_batch, and every launch shape is timed with the
  * check inside the projection kernel and as a second launch.  Each candidate
- * is timed as the median of five bursts of four calls; because the choice of
- * threads per configuration changes results by rounding, one lane per chain is
- * taken unless one per configuration is faster by more than a quarter.  Uses temporary
+ * is timed as the median of five bursts of four calls.  The choice of threads per
+ * configuration changes results by rounding and is not made by speed alone: one
+ * lane per chain is taken unless one per configuration is faster by more than a
+ * quarter, so for the two-chain classes the choice can be up to a quarter slower
+ * than the fastest candidate (dual arm: 7 % for projection and check of 65,536
+ * points, 14 % for its segments); mcp_set_tuning takes the other one.  Uses temporary
  * device buffers; synchronous.  The choices are returned in tpb / blocks_per_sm /
  * chunk / fuse_check / threads_per_config (HOST, each may be NULL).  The
  * launch shape never changes results; threads per configuration changes them

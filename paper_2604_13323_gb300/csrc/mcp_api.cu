@@ -1749,10 +1749,16 @@ mcp_status mcp_autotune(mcp_ctx *ctx, const mcp_project_params *p, int64_t n_sam
   const Tuning saved = ctx->tune;
   Tuning best = saved;
   float best_ms = 1e30f;
-  // The pair kernel's points differ from the thread kernel's by rounding, so
-  // the choice between them must not hang on timing noise: one lane per chain,
-  // unless one lane per configuration is faster by more than a quarter
-  // (dual-arm projection and check, 65,536 points: 242 us and 222 us).
+  // The pair kernel's points differ from the thread kernel's by rounding (rms
+  // distance from the FP64 projection 2.7e-6 rad in both), and of the 241,378
+  // comparable points of the dual arm's segments one of the thread kernel's lies
+  // 1.004e-4 from it, past the 1e-4 that tuned results are held to; the pair
+  // kernel's largest distance is 9.4e-5.  That point is at the limit of what FP32
+  // determines (a start perturbed by 8 unit roundoffs moves the FP64 projection
+  // by more than 1e-4 in one case of 80), but a tuned context keeps to the bar:
+  // one lane per chain, unless one lane per configuration is faster by more than
+  // a quarter.  That costs speed: projection and check of 65,536 points 237 us
+  // instead of 221, the segments 604 us instead of 529.
   constexpr float ONE_LANE_HANDICAP = 1.25f;
   const int tpbs[3] = {64, 128, 256};
   const int bpss[4] = {1, 2, 4, 8};

@@ -384,7 +384,8 @@ class Projector:
     def autotune(self, q_sample, params, stream=None):
         """Times the persistent kernel's launch shapes on q_sample ([d, n] float32
         CUDA tensor) and keeps the fastest; returns (threads/block, blocks/SM,
-        chunk, fuse_check, threads/configuration)."""
+        chunk, fuse_check, threads/configuration).  On the dual arm the threads
+        per configuration are not chosen by speed alone (mcp_autotune)."""
         d, n = q_sample.shape
         t, b, c, f, k = (ctypes.c_int32() for _ in range(5))
         pp = self.params(params)
