@@ -186,8 +186,9 @@ __device__ __forceinline__ void sincos_f64_table(double x, const double2 *__rest
 //   cos r - 1 = -r^2/2 + r^4/24      (first omitted term r^6/720 <= 2.0e-23)
 // the angle-addition formulas combine them.  The small terms are evaluated in
 // FP32, where their rounding lies far below that of the result: r^3/6 is at
-// most 2.0e-11, its FP32 error 2e-18; r^2/2 is carried as the rounded square
-// and its remainder.  6 FP64 operations (10 with the terms in FP64 and a table
+// most 2.0e-11, the four roundings of its evaluation 2^-22 of that, 5e-18; r^2/2
+// is carried as the rounded square and its remainder.  (In FP64 with |r| up to
+// 2^-10, as before, the omitted r^5/120 alone was 7.6e-18.)  6 FP64 operations (10 with the terms in FP64 and a table
 // of 512 per radian; an FP64 operation costs the SM 19 cycles, the FP32 ones
 // and the conversions together about 10).  Error against 64 bits over [-4, 4],
 // 2,000,000 angles: largest 1.79e-16, rms 4.6e-17 (sin), 4.9e-17 (cos); with the
@@ -196,16 +197,29 @@ __device__ __forceinline__ void sincos_f64_table(double x, const double2 *__rest
 constexpr int SPLIT_TAB_OFF = 256;   // entries [256, 256 + 8193): (sin, cos)(m / 1024), m = -4096..4096
 constexpr int SPLIT_TAB_HALF = 4096;
 constexpr float SPLIT_TAB_PER_RAD = 1024.f;
+__host__ __device__ __forceinline__ float mul_apart(float a, float b) {  // a product that is rounded, not contracted
+#ifdef __CUDA_ARCH__
+  return __fmul_rn(a, b);
+#else
+  volatile float p = a * b;
+  return p;
+#endif
+}
+// sin r and cos r - 1 for |r| <= 2^-11
+__host__ __device__ __forceinline__ void split_terms(float r, double &sr, double &cm) {
+  const float r2 = mul_apart(r, r), r2l = fmaf(r, r, -r2);  // r^2 = r2 + r2l
+  const float r3 = mul_apart(mul_apart(r, r2), -1.6666667e-1f);
+  const float cl = fmaf(-0.5f, r2l, mul_apart(mul_apart(r2, r2), 4.1666667e-2f));
+  sr = static_cast<double>(r) + static_cast<double>(r3);
+  cm = static_cast<double>(-0.5f * r2) + static_cast<double>(cl);
+}
 __device__ __forceinline__ void sincos_f64_split_f(float xf, const double2 *__restrict__ tab, double &s, double &c) {
   const float mf = rintf(xf * SPLIT_TAB_PER_RAD);
   if (fabsf(mf) <= static_cast<float>(SPLIT_TAB_HALF)) {
     const float r = fmaf(-mf, 1.f / SPLIT_TAB_PER_RAD, xf);  // exact
     const double2 t = __ldg(&tab[SPLIT_TAB_OFF + SPLIT_TAB_HALF + static_cast<int>(mf)]);
-    const float r2 = __fmul_rn(r, r), r2l = fmaf(r, r, -r2);  // r^2 = r2 + r2l
-    const float r3 = __fmul_rn(__fmul_rn(r, r2), -1.6666667e-1f);
-    const float cl = fmaf(-0.5f, r2l, __fmul_rn(__fmul_rn(r2, r2), 4.1666667e-2f));
-    const double sr = static_cast<double>(r) + static_cast<double>(r3);
-    const double cm = static_cast<double>(-0.5f * r2) + static_cast<double>(cl);
+    double sr, cm;
+    split_terms(r, sr, cm);
     s = fma(t.x, cm, fma(t.y, sr, t.x));
     c = fma(t.y, cm, fma(-t.x, sr, t.y));
   } else {
