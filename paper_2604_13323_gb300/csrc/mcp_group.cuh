@@ -1,5 +1,6 @@
-// Work plan of the humanoid's Newton step on four lanes, and the layout of one
-// configuration's state under it.
+// Reference of the order in which the humanoid's sums are taken, and of the
+// state a four-lane Newton step would keep: a work plan that the host checks
+// under tests/ build and compare with the library's kernel.  No kernel runs it.
 //
 // The plan fixes an order for every sum over joints: the limbs are assigned to
 // four lanes by longest-first scheduling and the trunk joints to the lane with
@@ -7,20 +8,18 @@
 // joints in ascending order, and the CoM sums in one partial per lane (the
 // lane's limb joints, then its trunk joints) added pairwise.  The projection
 // kernel (one lane per configuration, mcp_tree.cuh) takes its sums in this
-// order; the host checks under tests/ compile the plan and compare.  Also
-// here: the compile-time zero pattern of the Cholesky factor and the constants
-// of the floating base's prismatic chain, which that kernel uses.
+// order.  What that kernel uses itself is in mcp_factor.cuh.
 #pragma once
 
 #include <algorithm>
 #include <vector>
 
+#include "mcp_factor.cuh"
 #include "mcp_warp.cuh"
 
 namespace mcp {
 
-// Limits of the work plan (the plan is copied into every block's shared
-// memory, so they are kept near what the humanoid classes need).
+// Limits of the work plan, near what the humanoid classes need.
 constexpr int GG = 4;            // lanes per configuration
 constexpr int GCPW = 32 / GG;    // configurations per warp
 constexpr int GMAX_FK = 20;      // FK steps per lane
@@ -31,7 +30,7 @@ constexpr int GMAX_JI = 16;      // Jacobian segments per lane and segment size
 constexpr int GMAX_DQ = 20;      // dq joints per lane
 constexpr int GMAX_T = 2;        // Gram / refinement tasks per lane and phase
 constexpr int GMAX_POOL = 192;   // joint lists of the tasks
-constexpr int GMAX_PRE = 3;      // prismatic root joints placed in closed form
+constexpr int GMAX_PRE = PRE_JOINTS;  // prismatic root joints placed in closed form
 
 template <class P>
 __host__ __device__ constexpr bool grp_pose_like(int c) {
@@ -40,12 +39,6 @@ __host__ __device__ constexpr bool grp_pose_like(int c) {
 template <class P>
 __host__ __device__ constexpr bool grp_com_like(int c) {
   return P::ckind(c) == K_COM || P::ckind(c) == K_HULL;
-}
-template <class P>
-__host__ __device__ constexpr bool grp_supported() {
-  for (int c = 0; c < P::NC; ++c)
-    if (!grp_pose_like<P>(c) && !grp_com_like<P>(c)) return false;
-  return P::D <= 64 && kdim<P>() <= 4 * 5 && dfs_preorder<P>();
 }
 // Per-constraint data slots: the pose-like constraints (error frame G, point
 // x, log-map vector) and the support-hull ones (nearest-edge data) are stored
@@ -94,45 +87,6 @@ __host__ __device__ constexpr int lcol_base(int k) {
   int o = 0;
   for (int t = 0; t < k; ++t) o += K - t;
   return o;
-}
-
-// Structural nonzeros of the Cholesky factor of A = J J^T + lambda I, row by
-// row (bit b of row i: L[i][b] may be nonzero).  The symbolic factorisation:
-// L[i][b] is nonzero where A[i][b] is (rows i and b of J share a joint) or
-// where L[i][j] and L[b][j] are both nonzero for some column j < b.
-template <class P>
-__host__ __device__ constexpr uint32_t l_row_pattern(int row) {
-  constexpr int K = kdim<P>();
-  uint64_t jm[MAXK] = {};  // joints of row i of J
-  for (int i = 0; i < K; ++i)
-    for (int j = 0; j < P::D; ++j)
-      if (jnz<P>(i, j)) jm[i] |= uint64_t(1) << j;
-  uint32_t nz[MAXK] = {};
-  for (int i = 0; i < K; ++i)
-    for (int b = 0; b <= i; ++b) {
-      bool v = (b == i) || (jm[i] & jm[b]) != 0;
-      for (int j = 0; j < b && !v; ++j) v = ((nz[i] >> j) & 1u) != 0 && ((nz[b] >> j) & 1u) != 0;
-      if (v) nz[i] |= 1u << b;
-    }
-  return nz[row];
-}
-template <class P, int I>
-struct LRow {
-  static constexpr uint32_t value = l_row_pattern<P>(I);
-};
-// Rows 4 mm .. 4 mm + 3 (one per lane of a group) all lie below row k and
-// are structurally zero in column k of L: the group skips their update.
-template <class P, int MM, int KC>
-__host__ __device__ constexpr bool l_col_block_zero() {
-  constexpr uint32_t m = LRow<P, GG * MM>::value | LRow<P, GG * MM + 1>::value | LRow<P, GG * MM + 2>::value |
-                         LRow<P, GG * MM + 3>::value;
-  return GG * MM > KC && ((m >> KC) & 1u) == 0u;
-}
-// Columns 4 mm .. 4 mm + 3 all lie left of column k and row k of L is
-// structurally zero in them.
-template <class P, int KR, int MM>
-__host__ __device__ constexpr bool l_row_seg_zero() {
-  return GG * MM + GG - 1 < KR && ((LRow<P, KR>::value >> (GG * MM)) & 0xFu) == 0u;
 }
 
 // Tasks of the Gram build and of the refinement residual: row blocks (a, b)
@@ -493,10 +447,7 @@ struct GrpTables {
   float msub[P::D];
   int8_t rev[P::D];
   int8_t sgn[P::NC][P::D];  // column sign of joint j in constraint c
-  // the prismatic root chain in closed form (for its first GMAX_PRE joints):
-  // with q = 0 joint i's frame sits at pre_c[i] with rotation R_i; its axis
-  // is pre_a[i] = R_i e_z, so its origin is pre_c[i] + sum_{k <= i} q_k pre_a[k];
-  // pre_mc[i] = m_i R_i com_i; pre_R = the rotation after the last of them
+  // the prismatic root chain (PreChain)
   float pre_R[GMAX_PRE][9];
   float pre_a[GMAX_PRE][3];
   float pre_c[GMAX_PRE][3];
@@ -517,25 +468,13 @@ __host__ __device__ constexpr size_t grp_state_stride() {
 template <class P>
 GrpTables<P> make_grp_tables(const ModelT<float> &m, const ModelT<double> &m64) {
   GrpTables<P> t{};
-  {  // the prismatic root chain, in FP64 then rounded
-    double R[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1}, c[3] = {0, 0, 0};
-    for (int i = 0; i < GMAX_PRE && i < P::D && P::jtype(i) == PRIS && P::parent(i) == i - 1; ++i) {
-      const double *X = m64.X[i];
-      double Rn[9], cn[3];
-      for (int r = 0; r < 3; ++r) {
-        cn[r] = c[r] + R[r * 3] * X[3] + R[r * 3 + 1] * X[7] + R[r * 3 + 2] * X[11];
-        for (int cc = 0; cc < 3; ++cc)
-          Rn[r * 3 + cc] = R[r * 3] * X[cc] + R[r * 3 + 1] * X[4 + cc] + R[r * 3 + 2] * X[8 + cc];
-      }
-      for (int e = 0; e < 9; ++e) R[e] = Rn[e];
-      for (int r = 0; r < 3; ++r) c[r] = cn[r];
-      for (int e = 0; e < 9; ++e) t.pre_R[i][e] = static_cast<float>(R[e]);
-      for (int r = 0; r < 3; ++r) {
-        t.pre_a[i][r] = static_cast<float>(R[r * 3 + 2]);
-        t.pre_c[i][r] = static_cast<float>(c[r]);
-        t.pre_mc[i][r] = static_cast<float>(m64.mass[i] * (R[r * 3] * m64.com[i][0] + R[r * 3 + 1] * m64.com[i][1] +
-                                                           R[r * 3 + 2] * m64.com[i][2]));
-      }
+  const PreChain pc = make_pre_chain<P>(m64);
+  for (int i = 0; i < GMAX_PRE; ++i) {
+    for (int e = 0; e < 9; ++e) t.pre_R[i][e] = pc.R[i][e];
+    for (int r = 0; r < 3; ++r) {
+      t.pre_a[i][r] = pc.a[i][r];
+      t.pre_c[i][r] = pc.c[i][r];
+      t.pre_mc[i][r] = pc.mc[i][r];
     }
   }
   for (int j = 0; j < P::D; ++j) {

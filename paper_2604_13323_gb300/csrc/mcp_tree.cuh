@@ -40,7 +40,8 @@
 // do not depend on how lanes share the work.
 #pragma once
 
-#include "mcp_group.cuh"
+#include "mcp_factor.cuh"
+#include "mcp_group.cuh"  // only the order its host check compares with
 #include "mcp_pack.cuh"
 
 namespace mcp {
@@ -106,7 +107,7 @@ __host__ __device__ constexpr int tree_part(int j) {
   return base[j];
 }
 
-// Constants of the prismatic base chain (see GrpTables) and what follows from
+// Constants of the prismatic base chain (see PreChain) and what follows from
 // them, and the limbs' model data in left / right pairs.
 template <int N>
 struct TreeLimb {
@@ -172,7 +173,7 @@ void fill_limb(const ModelT<float> &m, int jl, int jr, int fl, int fr, TreeLimb<
 }
 template <class P>
 TreeConst<P> make_tree_const(const ModelT<float> &m, const ModelT<double> &m64) {
-  const GrpTables<P> g = make_grp_tables<P>(m, m64);
+  const PreChain g = make_pre_chain<P>(m64);
   TreeConst<P> t{};
   fill_limb(m, TR_LEG0, TR_LEG0 + TR_LEG, 0, 1, t.leg);
   fill_limb(m, TR_ARM0, TR_ARM0 + TR_ARM, 2, 3, t.arm);
@@ -185,12 +186,12 @@ TreeConst<P> make_tree_const(const ModelT<float> &m, const ModelT<double> &m64) 
     t.Qp[r] = make_float2(m.cQinv[0][4 * r + 3], m.cQinv[1][4 * r + 3]);
   }
   float jt[2][3][3], LL[2][6] = {}, CL[2][6] = {};
-  for (int e = 0; e < 9; ++e) t.R[e] = g.pre_R[2][e];
+  for (int e = 0; e < 9; ++e) t.R[e] = g.R[2][e];
   for (int i = 0; i < 3; ++i) {
     for (int r = 0; r < 3; ++r) {
-      t.a[i][r] = g.pre_a[i][r];
-      t.c[i][r] = g.pre_c[i][r];
-      t.mc[i][r] = g.pre_mc[i][r];
+      t.a[i][r] = g.a[i][r];
+      t.c[i][r] = g.c[i][r];
+      t.mc[i][r] = g.mc[i][r];
     }
     const float f = m.msub[i] * m.inv_mass;
     t.jc[i][0] = f * t.a[i][0];
