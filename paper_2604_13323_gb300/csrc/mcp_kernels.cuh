@@ -938,7 +938,8 @@ template <class P, typename T>
 struct CheckArgs {
   ModelT<T> m;
   SphereTable<T> st;
-  const T *obs;  // FP32: [n_obs * 8] (-2c, |c|^2 - r^2, -2r, pad) in the shifted frame; FP64: [n_obs * 4]
+  const T *obs;  // FP32: records of the shifted frame in pairs of 12 floats (obs_rec): obs_pairs(n_obs) of the
+                 // obstacles, then obs_pairs(obs_chunks(n_obs)) of their chunks; FP64: [n_obs * 4]
   const T *box;  // [n_box * 6] (FP32: shifted)
   int n_obs;
   int n_box;

@@ -11,13 +11,14 @@
 // (Four lanes per configuration, with the Jacobian, Gram matrix and factor in
 // shared memory, took 16,000 warp-instructions per iteration for 8
 // configurations.  Projection and check of 1,048,576 configurations 21.9 ms,
-// of 4,099 744 us, of 32 410 us; here 7.3 ms, 275 us and 140 us.)  Layout:
+// of 4,099 742 us, projection of 32 459 us; here, in turn with it on the same
+// device, 7.3 ms, 281 us and 153 us.)  Layout:
 //   * shared memory per configuration: 129 float2 (TREE_PAIRS), lane-major
 //     (pair e of lane l at [e * 32 + l]: conflict-free 64-bit accesses at
 //     immediate offsets); seven warps of 32 configurations fill an SM's 227 KB;
 //   * the left and the right leg, and the two arms, go through FK, Jacobian,
 //     Gram and solve together, two values per instruction (mcp_pack.cuh; with
-//     the limbs one after the other 7.2 ms instead of 6.5 ms);
+//     the limbs one after the other the projection took 6.9 ms instead of 6.2 ms);
 //   * Jacobian segments are built in loops over a limb's joints that fit the
 //     scheduler's own instruction buffer;
 //   * warps go through an iteration in step: a barrier between its phases
